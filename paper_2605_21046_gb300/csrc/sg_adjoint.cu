@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) k_bilinear(const BilinParams p) {
       double u[NKD];
 #pragma unroll
       for (int a = 0; a < NKD; ++a) u[a] = q[a];
-      forward_cell<F64, DIM, K>(u, q);
+      forward_cell<F64, DIM, K>(u, [&](int o, double v) { q[o] = v; });
     }
     __syncthreads();
     for (int it = tid; it < nc * NQD * n_xi; it += nthr) {
@@ -366,7 +366,7 @@ sg_status adjoint_gradient(sg_ctx* ctx, double rtol, int max_it, int K, int cell
   for (int d = 0; d < 3; ++d) {
     bp.nn[d] = hp.nn[d];
     bp.cells[d] = hp.cells[d];
-    bp.ratio[d] = d < hp.dim ? (hp.h[0] * hp.h[0]) / (hp.h[d] * hp.h[d]) : 0.0;
+    bp.ratio[d] = d < hp.dim ? grad_weight(hp.k) * (hp.h[0] * hp.h[0]) / (hp.h[d] * hp.h[d]) : 0.0;
   }
   bp.n_xi = hp.n_xi;
   bp.n_terms = hp.n_terms;

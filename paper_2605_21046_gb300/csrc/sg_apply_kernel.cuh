@@ -48,155 +48,309 @@ __device__ __forceinline__ typename A::T cdot(CF cf, XF xf) {
   return A::fin(s);
 }
 
+// --------------------------------------------------------------- 1D lines
+// The passes of the sum factorisation along one line of N = K + 1 values.
+//
+// Derivatives are taken in units of deriv_scale<K>(): with the Gauss points'
+// symmetry the collocation derivative needs few multiplies, and the remaining
+// common factor of every gradient is left out here and put back, squared, into
+// the coefficient (grad_weight<K>()), which multiplies each gradient once on
+// its way there and back.  FP64 instructions per line, dense tables against
+// this form: Q2 interpolation 6 / 6, derivative 8 / 4, their transposes 7 / 6
+// and 8 / 7, and 9 and 12 where one line needs value and derivative (15 and
+// 15); Q3 interpolation 16 / 14, derivative 16 / 12, transposes 16 / 14, both
+// at once 24 and 26 (32); Q1 derivative 4 / 2.  Double-word sums cost more than products (8 against
+// 4 instructions), so that arithmetic keeps the dense interpolation.  Bound by
+// the FP64 pipe (81 % active), the whole apply went from 186 to 165 us on 64^2
+// Q2 M=4 P=3, 3.36 to 3.02 ms on 32^3 Q2 M=3 P=3 and 1.79 to 1.62 ms on 128^2
+// Q3 dG(3); double-word 675 to 650 us on 128^2 Q2 M=4 P=4.  The error against
+// 64-bit references is the dense form's or less (Q2 4.5e-16 against 5.0e-16).
+template <int K>
+__host__ __device__ constexpr double deriv_scale() {
+  return K == 1 ? 1.0 : (K == 2 ? RefShape<2>::D(1, 2) : 0.5 * (RefShape<3>::D(3, 3) - RefShape<3>::D(3, 0)));
+}
+// deriv_scale squared: 1 (Q1 has one multiply to lose, and loses accuracy with
+// a rounded 3 a), 5/3, and the square of Q3's.
+template <int K>
+__host__ __device__ constexpr double grad_weight() {
+  return K == 1 ? 1.0 : (K == 2 ? 5.0 / 3.0 : deriv_scale<3>() * deriv_scale<3>());
+}
+__host__ __device__ constexpr double grad_weight(int k) {
+  return k == 1 ? 1.0 : (k == 2 ? grad_weight<2>() : grad_weight<3>());
+}
+__host__ __device__ constexpr Cf cf_of(double c) {
+  return {c, (float)c, (float)(c - (double)(float)c)};
+}
+
+template <class A, int K>
+struct Line {
+  using T = typename A::T;
+  static constexpr int N = K + 1;
+  template <class F>
+  static __device__ __forceinline__ void dense(F c, const T* x, T* y) {
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+      y[a] = cdot<A, N>([&](int j) { return c(a, j); }, [&](int j) { return x[j]; });
+  }
+  // c x + y for a compile-time c, as a sum still to be finished (A::fin)
+  static __device__ __forceinline__ T axpy(Cf c, T x, T y) {
+    A::cfma(c, x, y);
+    return y;
+  }
+  static __device__ __forceinline__ T axpy(double c, T x, T y) { return axpy(cf_of(c), x, y); }
+  static __device__ __forceinline__ T sub(T a, T b) { return A::add(a, A::neg(b)); }
+
+  // nodal values -> values at the Gauss points
+  static __device__ __forceinline__ void interp(const T (&u)[N], T (&v)[N]) {
+    if constexpr (A::kDW || K == 1) {
+      dense([](int a, int j) { return cS<K>(a, j); }, u, v);
+    } else if constexpr (K == 2) {
+      const T s = A::add(u[0], u[2]), d = sub(u[2], u[0]);
+      const T e = axpy(0.3, s, A::cmul(cf_of(0.4), u[1]));
+      v[0] = axpy(-kB2(), d, e);
+      v[1] = u[1];
+      v[2] = axpy(kB2(), d, e);
+    } else {
+      T eo, ei;
+      cubic(u, v, eo, ei);
+    }
+  }
+  // values at the Gauss points -> derivatives there, in units of deriv_scale
+  static __device__ __forceinline__ void deriv(const T (&v)[N], T (&g)[N]) {
+    if constexpr (K == 1) {
+      g[0] = g[1] = A::fin(axpy(cD<1>(1, 1), v[1], A::cmul(cD<1>(1, 0), v[0])));
+    } else if constexpr (K == 2) {
+      const T m = sub(v[2], v[0]), a = sub(v[2], v[1]);
+      const T p = axpy(4.0, a, A::neg(m));
+      g[0] = A::fin(axpy(2.0, m, A::neg(p)));
+      g[1] = A::fin(m);
+      g[2] = A::fin(p);
+    } else {
+      const T q = sub(A::add(v[0], v[3]), A::add(v[1], v[2]));
+      cubic_deriv(sub(v[3], v[0]), sub(v[2], v[1]), q, g);
+    }
+  }
+  // both at once (v as interp, g as deriv of v)
+  static __device__ __forceinline__ void interp_deriv(const T (&u)[N], T (&v)[N], T (&g)[N]) {
+    if constexpr (!A::kDW && K == 2) {
+      const T s = A::add(u[0], u[2]), d = sub(u[2], u[0]);
+      const T t = axpy(-2.0, u[1], s);
+      const T e = axpy(0.3, t, u[1]), m = A::cmul(cf_of(2.0 * kB2()), d);
+      v[0] = axpy(-0.5, m, e);
+      v[1] = u[1];
+      v[2] = axpy(0.5, m, e);
+      g[0] = axpy(-1.2, t, m);
+      g[1] = m;
+      g[2] = axpy(1.2, t, m);
+    } else if constexpr (!A::kDW && K == 3) {
+      T eo, ei;
+      cubic(u, v, eo, ei);
+      const T q = sub(eo, ei);
+      cubic_deriv(sub(v[3], v[0]), sub(v[2], v[1]), A::add(q, q), g);
+    } else {
+      interp(u, v);
+      deriv(v, g);
+    }
+  }
+  // r += transpose of deriv applied to g (sums still to be finished)
+  static __device__ __forceinline__ void deriv_t(const T (&g)[N], T (&r)[N]) {
+    if constexpr (K == 1) {
+      const T G = A::add(g[0], g[1]);
+      r[0] = axpy(cD<1>(0, 0), G, r[0]);
+      r[1] = axpy(cD<1>(0, 1), G, r[1]);
+    } else if constexpr (K == 2) {
+      const T P = sub(g[2], g[0]);
+      const T B = sub(axpy(2.0, g[0], g[1]), P);   // the odd part: -B on one end, B + 4 P on the other
+      r[0] = sub(r[0], B);
+      r[1] = axpy(-4.0, P, r[1]);
+      r[2] = axpy(4.0, P, A::add(r[2], B));
+    } else {
+#pragma unroll
+      for (int a = 0; a < N; ++a)
+#pragma unroll
+        for (int j = 0; j < N; ++j) r[a] = axpy(RefShape<3>::D(j, a) / deriv_scale<3>(), g[j], r[a]);
+    }
+  }
+  // transpose of interp
+  static __device__ __forceinline__ void interp_t(const T (&r)[N], T (&n)[N]) {
+    if constexpr (A::kDW || K == 1) {
+      dense([](int a, int j) { return cS<K>(j, a); }, r, n);
+    } else if constexpr (K == 2) {
+      quad_t(A::add(r[0], r[2]), sub(r[2], r[0]), r[1], n);
+    } else {
+      cubic_t(A::add(r[0], r[3]), A::add(r[1], r[2]), sub(r[3], r[0]), sub(r[2], r[1]), n);
+    }
+  }
+  // n = transpose of interp applied to (r + transpose of deriv applied to g)
+  static __device__ __forceinline__ void interp_deriv_t(T (&r)[N], const T (&g)[N], T (&n)[N]) {
+    if constexpr (!A::kDW && K == 2) {
+      const T P = sub(g[2], g[0]), S = A::add(A::add(g[0], g[2]), g[1]);
+      quad_t(axpy(4.0, P, A::add(r[0], r[2])), axpy(2.0, S, sub(r[2], r[0])), axpy(-4.0, P, r[1]), n);
+    } else if constexpr (!A::kDW && K == 3) {
+      const T Go = A::add(g[0], g[3]), Gi = A::add(g[1], g[2]), Ho = sub(g[3], g[0]), Hi = sub(g[2], g[1]);
+      const T Q = axpy(2.0 * kQo(), Ho, A::cmul(cf_of(2.0 * kQi()), Hi));
+      const T so = A::add(A::add(r[0], r[3]), Q), si = sub(A::add(r[1], r[2]), Q);
+      const T dO = axpy(2.0 * kAi(), Gi, axpy(2.0, Go, sub(r[3], r[0])));
+      const T dI = axpy(2.0 * kBi(), Gi, axpy(2.0 * kBo(), Go, sub(r[2], r[1])));
+      cubic_t(so, si, dO, dI, n);
+    } else {
+      deriv_t(g, r);
+#pragma unroll
+      for (int a = 0; a < N; ++a) r[a] = A::fin(r[a]);
+      interp_t(r, n);
+    }
+  }
+
+ private:
+  // Q2: half the difference of the end functions at the outer Gauss point (sqrt(3/5) / 2);
+  // their mean there is 0.3, the middle function 0.4
+  static __host__ __device__ constexpr double kB2() { return 0.5 * (RefShape<2>::S(2, 2) - RefShape<2>::S(2, 0)); }
+  static __device__ __forceinline__ void quad_t(T s, T o, T r1, T (&n)[N]) {
+    const T t = A::cmul(cf_of(0.3), s);
+    n[0] = axpy(-kB2(), o, t);
+    n[1] = axpy(0.4, s, r1);
+    n[2] = axpy(kB2(), o, t);
+  }
+  // Q3: even (E) and odd (C) parts of the end (0) and inner (1) basis functions at the outer (o) and
+  // inner (i) Gauss points, and the derivative's weights on (v3 - v0), (v2 - v1) and (v0 + v3) - (v1 + v2)
+  static __host__ __device__ constexpr double sE(int q, int n) { return 0.5 * (RefShape<3>::S(q, n) + RefShape<3>::S(q, 3 - n)); }
+  static __host__ __device__ constexpr double sC(int q, int n) { return 0.5 * (RefShape<3>::S(q, n) - RefShape<3>::S(q, 3 - n)); }
+  static __host__ __device__ constexpr double kQo() { return 0.5 * (RefShape<3>::D(3, 3) + RefShape<3>::D(3, 0)) / deriv_scale<3>(); }
+  static __host__ __device__ constexpr double kQi() { return 0.5 * (RefShape<3>::D(2, 3) + RefShape<3>::D(2, 0)) / deriv_scale<3>(); }
+  static __host__ __device__ constexpr double kAi() { return 0.5 * (RefShape<3>::D(2, 3) - RefShape<3>::D(2, 0)) / deriv_scale<3>(); }
+  static __host__ __device__ constexpr double kBo() { return 0.5 * (RefShape<3>::D(3, 2) - RefShape<3>::D(3, 1)) / deriv_scale<3>(); }
+  static __host__ __device__ constexpr double kBi() { return 0.5 * (RefShape<3>::D(2, 2) - RefShape<3>::D(2, 1)) / deriv_scale<3>(); }
+  static __device__ __forceinline__ void cubic(const T (&u)[N], T (&v)[N], T& eo, T& ei) {
+    const T s0 = A::add(u[0], u[3]), s1 = A::add(u[1], u[2]), d0 = sub(u[3], u[0]), d1 = sub(u[2], u[1]);
+    eo = axpy(sE(3, 2), s1, A::cmul(cf_of(sE(3, 3)), s0));
+    ei = axpy(sE(2, 2), s1, A::cmul(cf_of(sE(2, 3)), s0));
+    const T wo = axpy(sC(3, 2) / sC(3, 3), d1, d0), wi = axpy(sC(2, 3) / sC(2, 2), d0, d1);
+    v[0] = axpy(-sC(3, 3), wo, eo);
+    v[1] = axpy(-sC(2, 2), wi, ei);
+    v[2] = axpy(sC(2, 2), wi, ei);
+    v[3] = axpy(sC(3, 3), wo, eo);
+  }
+  static __device__ __forceinline__ void cubic_deriv(T d0, T d1, T q, T (&g)[N]) {
+    const T eo = axpy(kBo(), d1, d0), ei = axpy(kBi(), d1, A::cmul(cf_of(kAi()), d0));
+    g[0] = A::fin(axpy(-kQo(), q, eo));
+    g[1] = A::fin(axpy(-kQi(), q, ei));
+    g[2] = A::fin(axpy(kQi(), q, ei));
+    g[3] = A::fin(axpy(kQo(), q, eo));
+  }
+  static __device__ __forceinline__ void cubic_t(T so, T si, T dO, T dI, T (&n)[N]) {
+    const T n0 = axpy(sE(2, 3), si, A::cmul(cf_of(sE(3, 3)), so)), n1 = axpy(sE(2, 2), si, A::cmul(cf_of(sE(3, 2)), so));
+    const T x0 = axpy(sC(2, 3) / sC(3, 3), dI, dO), x1 = axpy(sC(3, 2) / sC(2, 2), dO, dI);
+    n[0] = axpy(-sC(3, 3), x0, n0);
+    n[1] = axpy(-sC(2, 2), x1, n1);
+    n[2] = axpy(sC(2, 2), x1, n1);
+    n[3] = axpy(sC(3, 3), x0, n0);
+  }
+};
+
+// Line i (of the others, counted in order) along direction d of an N^DIM
+// array, x fastest: its first entry and its stride.
+template <int N>
+__host__ __device__ constexpr int line_stride(int d) {
+  return d == 0 ? 1 : (d == 1 ? N : N * N);
+}
+template <int N>
+__host__ __device__ constexpr int line_first(int d, int i) {
+  return d == 0 ? i * N : (d == 1 ? (i / N) * N * N + i % N : i);
+}
+
 // --------------------------------------------------------------- phase 1
 // Nodal values u (lexicographic, x fastest) -> values and reference gradients
-// at the tensor Gauss points, written to q[comp * NQD + point].
-template <class A, int DIM, int K>
-__device__ __forceinline__ void forward_cell(const typename A::T* u, typename A::T* q) {
+// (in units of deriv_scale) at the tensor Gauss points: x, then y (, then z)
+// interpolation in place, the last direction with its derivative; the other
+// derivatives by collocation.  put(comp * NQD + point, value) stores them.
+template <class A, int DIM, int K, class Put>
+__device__ __forceinline__ void forward_cell(typename A::T* u, Put put) {
   using T = typename A::T;
-  using Sh = Shape<DIM, K>;
-  constexpr int N = Sh::N;
-  constexpr Cf one = {1.0, 1.0f, 0.0f};
-  (void)one;
-  if constexpr (DIM == 2) {
-    T t[N][N];   // [ny][qx]
+  using L = Line<A, K>;
+  constexpr int N = K + 1, NQD = Shape<DIM, K>::NQD, NL = NQD / N;
+  T in[N], v[N], g[N];
 #pragma unroll
-    for (int ny = 0; ny < N; ++ny)
+  for (int d = 0; d < DIM; ++d) {
+    const int st = line_stride<N>(d);
 #pragma unroll
-      for (int qx = 0; qx < N; ++qx)
-        t[ny][qx] = cdot<A, N>([&](int j) { return cS<K>(qx, j); }, [&](int j) { return u[ny * N + j]; });
-    T v[N][N];   // [qy][qx]
+    for (int i = 0; i < NL; ++i) {
+      const int o = line_first<N>(d, i);
 #pragma unroll
-    for (int qy = 0; qy < N; ++qy)
+      for (int j = 0; j < N; ++j) in[j] = u[o + j * st];
+      if (d + 1 < DIM) {
+        L::interp(in, v);
+      } else {
+        L::interp_deriv(in, v, g);
 #pragma unroll
-      for (int qx = 0; qx < N; ++qx) {
-        v[qy][qx] = cdot<A, N>([&](int j) { return cS<K>(qy, j); }, [&](int j) { return t[j][qx]; });
-        q[qy * N + qx] = v[qy][qx];
+        for (int j = 0; j < N; ++j) put((1 + d) * NQD + o + j * st, g[j]);
       }
 #pragma unroll
-    for (int qy = 0; qy < N; ++qy)
-#pragma unroll
-      for (int qx = 0; qx < N; ++qx) {
-        q[Sh::NQD + qy * N + qx] = cdot<A, N>([&](int r) { return cD<K>(qx, r); }, [&](int r) { return v[qy][r]; });
-        q[2 * Sh::NQD + qy * N + qx] = cdot<A, N>([&](int r) { return cD<K>(qy, r); }, [&](int r) { return v[r][qx]; });
+      for (int j = 0; j < N; ++j) {
+        u[o + j * st] = v[j];
+        if (d + 1 == DIM) put(o + j * st, v[j]);
       }
-  } else {
-    T t1[N][N][N];  // [nz][ny][qx]
+    }
+  }
 #pragma unroll
-    for (int nz = 0; nz < N; ++nz)
+  for (int d = 0; d + 1 < DIM; ++d) {
+    const int st = line_stride<N>(d);
 #pragma unroll
-      for (int ny = 0; ny < N; ++ny)
+    for (int i = 0; i < NL; ++i) {
+      const int o = line_first<N>(d, i);
 #pragma unroll
-        for (int qx = 0; qx < N; ++qx)
-          t1[nz][ny][qx] = cdot<A, N>([&](int j) { return cS<K>(qx, j); },
-                                      [&](int j) { return u[(nz * N + ny) * N + j]; });
-    T t2[N][N][N];  // [nz][qy][qx]
+      for (int j = 0; j < N; ++j) in[j] = u[o + j * st];
+      L::deriv(in, g);
 #pragma unroll
-    for (int nz = 0; nz < N; ++nz)
-#pragma unroll
-      for (int qy = 0; qy < N; ++qy)
-#pragma unroll
-        for (int qx = 0; qx < N; ++qx)
-          t2[nz][qy][qx] = cdot<A, N>([&](int j) { return cS<K>(qy, j); }, [&](int j) { return t1[nz][j][qx]; });
-    T v[N][N][N];   // [qz][qy][qx]
-#pragma unroll
-    for (int qz = 0; qz < N; ++qz)
-#pragma unroll
-      for (int qy = 0; qy < N; ++qy)
-#pragma unroll
-        for (int qx = 0; qx < N; ++qx) {
-          v[qz][qy][qx] = cdot<A, N>([&](int j) { return cS<K>(qz, j); }, [&](int j) { return t2[j][qy][qx]; });
-          q[(qz * N + qy) * N + qx] = v[qz][qy][qx];
-        }
-#pragma unroll
-    for (int qz = 0; qz < N; ++qz)
-#pragma unroll
-      for (int qy = 0; qy < N; ++qy)
-#pragma unroll
-        for (int qx = 0; qx < N; ++qx) {
-          const int o = (qz * N + qy) * N + qx;
-          q[Sh::NQD + o] = cdot<A, N>([&](int r) { return cD<K>(qx, r); }, [&](int r) { return v[qz][qy][r]; });
-          q[2 * Sh::NQD + o] = cdot<A, N>([&](int r) { return cD<K>(qy, r); }, [&](int r) { return v[qz][r][qx]; });
-          q[3 * Sh::NQD + o] = cdot<A, N>([&](int r) { return cD<K>(qz, r); }, [&](int r) { return v[r][qy][qx]; });
-        }
+      for (int j = 0; j < N; ++j) put((1 + d) * NQD + o + j * st, g[j]);
+    }
   }
 }
 
 // --------------------------------------------------------------- phase 3
-// Point values (q[0..NQD)) and reference-gradient coefficients
-// (q[NQD*(1+d) ...]) -> nodal contributions, written over q[0..NKD).  All
-// reads of q happen before the first write.
-template <class A, int DIM, int K>
-__device__ __forceinline__ void backward_cell(typename A::T* q) {
+// Point values and reference-gradient coefficients (get(comp * NQD + point))
+// -> nodal contributions r: the transpose of forward_cell.
+template <class A, int DIM, int K, class Get>
+__device__ __forceinline__ void backward_cell(Get get, typename A::T* r) {
   using T = typename A::T;
-  using Sh = Shape<DIM, K>;
-  constexpr int N = Sh::N;
-  constexpr Cf one = {1.0, 1.0f, 0.0f};
-  if constexpr (DIM == 2) {
-    T r[N][N];   // [qy][qx] combined point residual
+  using L = Line<A, K>;
+  constexpr int N = K + 1, NQD = Shape<DIM, K>::NQD, NL = NQD / N;
+  T in[N], g[N], out[N];
 #pragma unroll
-    for (int qy = 0; qy < N; ++qy)
+  for (int q = 0; q < NQD; ++q) r[q] = get(q);
 #pragma unroll
-      for (int qx = 0; qx < N; ++qx)
-        r[qy][qx] = cdot<A, 2 * N + 1>(
-            [&](int j) { return j == 0 ? one : (j <= N ? cD<K>(j - 1, qx) : cD<K>(j - 1 - N, qy)); },
-            [&](int j) {
-              return j == 0 ? q[qy * N + qx]
-                            : (j <= N ? q[Sh::NQD + qy * N + (j - 1)] : q[2 * Sh::NQD + (j - 1 - N) * N + qx]);
-            });
-    T t[N][N];   // [ny][qx]
+  for (int d = 0; d + 1 < DIM; ++d) {
+    const int st = line_stride<N>(d);
 #pragma unroll
-    for (int ny = 0; ny < N; ++ny)
+    for (int i = 0; i < NL; ++i) {
+      const int o = line_first<N>(d, i);
 #pragma unroll
-      for (int qx = 0; qx < N; ++qx)
-        t[ny][qx] = cdot<A, N>([&](int j) { return cS<K>(j, ny); }, [&](int j) { return r[j][qx]; });
+      for (int j = 0; j < N; ++j) {
+        in[j] = r[o + j * st];
+        g[j] = get((1 + d) * NQD + o + j * st);
+      }
+      L::deriv_t(g, in);
 #pragma unroll
-    for (int ny = 0; ny < N; ++ny)
+      for (int j = 0; j < N; ++j) r[o + j * st] = in[j];
+    }
+  }
 #pragma unroll
-      for (int nx = 0; nx < N; ++nx)
-        q[ny * N + nx] = cdot<A, N>([&](int j) { return cS<K>(j, nx); }, [&](int j) { return t[ny][j]; });
-  } else {
-    T r[N][N][N];
+  for (int d = DIM - 1; d >= 0; --d) {
+    const int st = line_stride<N>(d);
 #pragma unroll
-    for (int qz = 0; qz < N; ++qz)
+    for (int i = 0; i < NL; ++i) {
+      const int o = line_first<N>(d, i);
 #pragma unroll
-      for (int qy = 0; qy < N; ++qy)
+      for (int j = 0; j < N; ++j) in[j] = r[o + j * st];
+      if (d + 1 == DIM) {
 #pragma unroll
-        for (int qx = 0; qx < N; ++qx)
-          r[qz][qy][qx] = cdot<A, 3 * N + 1>(
-              [&](int j) {
-                return j == 0 ? one
-                              : (j <= N ? cD<K>(j - 1, qx) : (j <= 2 * N ? cD<K>(j - 1 - N, qy) : cD<K>(j - 1 - 2 * N, qz)));
-              },
-              [&](int j) {
-                return j == 0 ? q[(qz * N + qy) * N + qx]
-                              : (j <= N ? q[Sh::NQD + (qz * N + qy) * N + (j - 1)]
-                                        : (j <= 2 * N ? q[2 * Sh::NQD + (qz * N + (j - 1 - N)) * N + qx]
-                                                      : q[3 * Sh::NQD + ((j - 1 - 2 * N) * N + qy) * N + qx]));
-              });
-    T t1[N][N][N];  // [nz][qy][qx]
+        for (int j = 0; j < N; ++j) g[j] = get((1 + d) * NQD + o + j * st);
+        L::interp_deriv_t(in, g, out);
+      } else {
+        L::interp_t(in, out);
+      }
 #pragma unroll
-    for (int nz = 0; nz < N; ++nz)
-#pragma unroll
-      for (int qy = 0; qy < N; ++qy)
-#pragma unroll
-        for (int qx = 0; qx < N; ++qx)
-          t1[nz][qy][qx] = cdot<A, N>([&](int j) { return cS<K>(j, nz); }, [&](int j) { return r[j][qy][qx]; });
-    T t2[N][N][N];  // [nz][ny][qx]
-#pragma unroll
-    for (int nz = 0; nz < N; ++nz)
-#pragma unroll
-      for (int ny = 0; ny < N; ++ny)
-#pragma unroll
-        for (int qx = 0; qx < N; ++qx)
-          t2[nz][ny][qx] = cdot<A, N>([&](int j) { return cS<K>(j, ny); }, [&](int j) { return t1[nz][j][qx]; });
-#pragma unroll
-    for (int nz = 0; nz < N; ++nz)
-#pragma unroll
-      for (int ny = 0; ny < N; ++ny)
-#pragma unroll
-        for (int nx = 0; nx < N; ++nx)
-          q[(nz * N + ny) * N + nx] = cdot<A, N>([&](int j) { return cS<K>(j, nx); }, [&](int j) { return t2[nz][ny][j]; });
+      for (int j = 0; j < N; ++j) r[o + j * st] = out[j];
+    }
   }
 }
 
@@ -258,11 +412,11 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
 
   if (premul) {
     for (int k = tid; k < p.n_pairs; k += nthr) {
-      Gv[k] = A::in(p.pair_val[k]);
+      Gv[k] = A::in(p.pair_val[k] * grad_weight<K>());
       Pt[k] = p.pair_term[k];
     }
   } else {
-    for (int e = tid; e < p.nnz; e += nthr) Gv[e] = A::in(p.g_val[e]);
+    for (int e = tid; e < p.nnz; e += nthr) Gv[e] = A::in(p.g_val[e] * grad_weight<K>());
   }
   for (int e = tid; e < p.nnz; e += nthr) {
     CoupleEntry ce;
@@ -299,8 +453,8 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
     {
       const int per_cell = p.n_terms * NQD;
       if (premul) {
-        // G value x a_term(x_q) per (cell, pair, point), rounded exactly as the
-        // product at the Gauss point would be
+        // G value x a_term(x_q) per (cell, pair, point); the G values carry the
+        // gradients' common factor (grad_weight)
         const int per_row = rows * NQD;
         for (int idx = tid; idx < nc * per_row; idx += nthr) {
           const int c = idx / per_row, r = idx - c * per_row;
@@ -360,7 +514,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
       T u[NKD];
 #pragma unroll
       for (int a = 0; a < NKD; ++a) u[a] = q[a];
-      forward_cell<A, DIM, K>(u, q);
+      forward_cell<A, DIM, K>(u, [&](int o, T v) { q[o] = v; });
     }
     __syncthreads();
     // ---------------------------------------------------------- phase 2
@@ -423,7 +577,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
                   const int ee = -1 - ce.tq;
                   const long long at = (c0 + c) * p.n_terms * NQD + p.g_term[ee] * NQD + q;
                   const double a_q = SG_IN(at, p.n_cells * p.n_terms * NQD, 108) ? p.ctab[at] : 0.0;
-                  couple(A::fin(A::mul(A::in(p.g_val[ee]), A::in(a_q))), ce.off);
+                  couple(A::fin(A::mul(A::in(p.g_val[ee] * grad_weight<K>()), A::in(a_q))), ce.off);
                 }
               }
             } else {
@@ -455,7 +609,13 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
     }
     __syncthreads();
     // ---------------------------------------------------------- phase 3
-    for (int it = tid; it < nc * V; it += nthr) backward_cell<A, DIM, K>(Qs + (size_t)it * SLOT);
+    for (int it = tid; it < nc * V; it += nthr) {
+      T* q = Qs + (size_t)it * SLOT;
+      T r[NKD];
+      backward_cell<A, DIM, K>([&](int o) { return q[o]; }, r);
+#pragma unroll
+      for (int a = 0; a < NKD; ++a) q[a] = r[a];
+    }
     __syncthreads();
     // ---------------------------------------------------------- phase 4
     for (int c = 0; c < nc; ++c) {

@@ -105,6 +105,7 @@ struct DW {
   __device__ __forceinline__ static T cmul(Cf c, T x) {
     if (c.c == 1.0) return x;
     if (c.c == -1.0) return {-x.h, -x.l};
+    if (c.c == 2.0 || c.c == -2.0 || c.c == 4.0 || c.c == -4.0) return {c.h * x.h, c.h * x.l};   // exact
     const float p = __fmul_rn(c.h, x.h);
     float e = __fmaf_rn(c.h, x.h, -p);
     e = __fmaf_rn(c.h, x.l, e);

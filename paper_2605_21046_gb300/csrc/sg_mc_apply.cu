@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) mc_apply_kernel(const McParams p) {
     const int nnx = P.nn[0], nny = P.nn[1], nnz_ = P.nn[2];
     __syncthreads();   // the previous chunk is done with shared memory
     if (pi != cur_prob || tile != cur_tile) {
-      for (int e = tid; e < ns * nterm; e += nthr) Wt[e] = A::in(P.wgt[(size_t)s0 * nterm + e]);
+      for (int e = tid; e < ns * nterm; e += nthr) Wt[e] = A::in(P.wgt[(size_t)s0 * nterm + e] * grad_weight<K>());
       if (pi != cur_prob)
         for (int e = tid; e < NQD * NT * NT; e += nthr) Amq[e] = A::in(P.amq[e]);
       cur_prob = pi;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) mc_apply_kernel(const McParams p) {
       T uv[NKD];
 #pragma unroll
       for (int a = 0; a < NKD; ++a) uv[a] = q[a];
-      forward_cell<A, DIM, K>(uv, q);
+      forward_cell<A, DIM, K>(uv, [&](int o, T v) { q[o] = v; });
     }
     __syncthreads();
     // phase 2: per (cell, point, sample): mass coupling and a(x_q, xi_s) grad u.
@@ -182,7 +182,13 @@ __global__ void __launch_bounds__(256) mc_apply_kernel(const McParams p) {
     }
     __syncthreads();
     // phase 3: back to the nodes
-    for (int it = tid; it < nc * VT; it += nthr) backward_cell<A, DIM, K>(Qs + (size_t)it * SLOT);
+    for (int it = tid; it < nc * VT; it += nthr) {
+      T* q = Qs + (size_t)it * SLOT;
+      T r[NKD];
+      backward_cell<A, DIM, K>([&](int o) { return q[o]; }, r);
+#pragma unroll
+      for (int a = 0; a < NKD; ++a) q[a] = r[a];
+    }
     __syncthreads();
     // phase 4: scale by tau Bhat_ii and add into y
     for (int c = 0; c < nc; ++c) {
