@@ -198,6 +198,27 @@ cudaError_t prepare_mc_kernel(int precision, int dim, int k, int n_t);
 // Precision of the apply kernels used inside the multigrid preconditioner.
 constexpr int kPrecF32 = SG_PREC_FP32;
 
+// ---------------------------------------------------------------- row-diagonal apply
+// y += sign * (T (x) M + B_t (x) K[sum_t wgt[row][t] a_t]) x_row for every row;
+// Dirichlet nodes are read as 0 and not written (sg_diag.cu).
+struct DiagParams {
+  const void* x;             // rows x N_t x n_x (float or double)
+  void* y;
+  const void* ctab;          // diag_coefficients' table
+  const void* wgt;           // [rows][n_terms] in the precision of the vectors
+  const double* amq;         // HOST [NQD][N_t][N_t]: w_q |J| T[i][j] / (tau Bhat_ii)
+  double sign;
+  long long n_x;
+  int n_cells, rows, n_terms, mass_only;
+  int cells[3], nn[3];
+  double ratio[3], tb[kMaxNT];
+};
+cudaError_t launch_diag_apply(int precision, int dim, int k, int n_t, const DiagParams& p, cudaStream_t s);
+// The coefficient of the terms `used` as [term][NQD][cell] in the given
+// precision (allocates *out; synchronous).
+cudaError_t diag_coefficients(int precision, const HostProblem& hp, const double* d_ctab, const std::vector<int>& used,
+                              void** out, cudaStream_t s);
+
 // ---------------------------------------------------------------- multigrid
 struct MGLevel {
   HostProblem hp;            // level discretisation; hp.g holds the diagonal (block-Jacobi) coupling
@@ -211,13 +232,10 @@ struct MGLevel {
   int* d_gterm = nullptr;
   double* d_gval = nullptr;
   int* d_perm = nullptr;
-  double* d_amq = nullptr;   // time-mass tables of the level's diagonal apply (A_t and A_t^T)
-  double* d_amqT = nullptr;
-  int mc_ts = 0;             // rows per tile of the level's diagonal apply
-  bool use_diag = true;      // residual by the diagonal apply (else the SG cell kernel, ls)
+  std::vector<double> amq[2];          // time-mass tables of the row-diagonal apply (A_t and A_t^T)
+  void* d_coef = nullptr;    // coefficient of the row-diagonal apply, [used term][point][cell]
+  bool use_diag = true;      // residual by the row-diagonal apply (else the SG cell kernel, ls)
   bool chunk_ok = false;     // the SG cell kernel has a launch shape for this level
-  int mc_chunk = 0, mc_grid = 0, mc_threads = 256;
-  size_t mc_smem = 0;
   void* d_inv = nullptr;     // [class][cell][np][pitch] patch inverses (pitch = np rounded up to 8;
                              //  bf16 when MG::bf16), or coarsest [class][n_int][n_int]
   int vanka_chunk = 0;       // cells per Vanka chunk
@@ -257,9 +275,9 @@ struct MG {
   bool bf16 = false;              // patch inverses stored in bf16 (FP32 vectors)
   int n_blk = 0;                  // Vanka mode blocks (modes of one class)
   int vanka_tile = 0;             // modes per Vanka tile (all of them unless Monte-Carlo)
-  bool mc = false;                // rows are Monte-Carlo samples: residuals by the MC apply
-  int mc_ts = 0;                  // samples per tile of the MC apply
-  double* d_wgt = nullptr;        // [S][n_terms] Psi_t(xi_s)
+  bool mc = false;                // rows are Monte-Carlo samples
+  std::vector<int> used;          // coefficient terms with a nonzero weight in any row
+  void* d_wused = nullptr;        // [rows][used] their weights in the MG precision
   int* d_blk_cls = nullptr;
   int* d_blk_alpha = nullptr;
   int nu = 2;
@@ -282,10 +300,8 @@ struct MG {
 sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega, MG& mg, std::string& msg,
                    bool single_class = false);
 // The mean-operator V-cycle of a Monte-Carlo system whose rows are samples
-// (weights [S][n_terms]): level residuals use the Monte-Carlo apply with ts
-// samples per tile, the Vanka smoother works in tiles of vanka_tile samples.
-sg_status mg_build_mc(const HostProblem& fine, int precision, int nu, double omega, const std::vector<double>& wgt,
-                      int ts, MG& mg, std::string& msg);
+// (hp.g holds their weights): the Vanka smoother works in tiles of vanka_tile samples.
+sg_status mg_build_mc(const HostProblem& fine, int precision, int nu, double omega, MG& mg, std::string& msg);
 size_t krylov_bytes(long long N, int m);
 void mg_free(MG& mg);
 // Per-level choices of a built multigrid: info = {levels, cells, coarsest,

@@ -211,8 +211,7 @@ __global__ void __launch_bounds__(256) mc_apply_kernel(const McParams p) {
 void* select_mc(int precision, int dim, int k, int n_t) {
 #define SG_M(D, KK, TT)                                                                              \
   if (dim == D && k == KK && n_t == TT)                                                              \
-    return precision == kPrecF32 ? reinterpret_cast<void*>(&mc_apply_kernel<F32, D, KK, TT>)         \
-                                 : reinterpret_cast<void*>(&mc_apply_kernel<F64, D, KK, TT>);
+    return reinterpret_cast<void*>(&mc_apply_kernel<F64, D, KK, TT>);
   SG_M(2, 1, 1) SG_M(2, 1, 2) SG_M(2, 1, 3) SG_M(2, 1, 4)
   SG_M(2, 2, 1) SG_M(2, 2, 2) SG_M(2, 2, 3) SG_M(2, 2, 4)
   SG_M(2, 3, 1) SG_M(2, 3, 2) SG_M(2, 3, 3) SG_M(2, 3, 4)

@@ -4,9 +4,8 @@
 //     A_alpha = A_t (x) M_x + sum_mu [G_mu]_{alpha alpha} B_t (x) K_mu,
 // with a space-time Vanka patch smoother.  All N_xi * N_t vectors go through
 // the V-cycle together, so one launch smooths every mode.  A level residual is
-// either the SG cell kernel with the diagonal coupling table or the diagonal
-// (Monte-Carlo) apply with per-row weights [G_mu]_{alpha alpha}; set-up times
-// both on the level and keeps the faster.
+// the row-diagonal apply with per-row weights [G_mu]_{alpha alpha} (sg_diag.cu)
+// or the SG cell kernel with the diagonal coupling table.
 //
 // Levels halve the cells per direction while every count is even and > 2;
 // coefficients are re-evaluated on every level (a per-cell scale is averaged
@@ -831,68 +830,48 @@ std::vector<double> coarsen_scale(const std::vector<double>& s, const HostProble
 template <typename T>
 cudaError_t issue_vcycle(MG& mg, int l, cudaStream_t s, int trans);
 
+// r -= A x inside by the row-diagonal apply (r holds b inside and 0 on the boundary)
+cudaError_t diag_residual(MG& mg, MGLevel& L, cudaStream_t s, int trans) {
+  DiagParams q;
+  std::memset(&q, 0, sizeof(q));
+  q.x = L.d_x;
+  q.y = L.d_r;
+  q.ctab = L.d_coef;
+  q.wgt = mg.d_wused;
+  q.amq = L.amq[trans ? 1 : 0].data();
+  q.sign = -1.0;
+  q.n_x = L.hp.n_x;
+  q.n_cells = (int)L.hp.n_cells;
+  q.rows = L.hp.n_xi;
+  q.n_terms = (int)mg.used.size();
+  for (int d = 0; d < 3; ++d) {
+    q.nn[d] = L.hp.nn[d];
+    q.cells[d] = L.hp.cells[d];
+    q.ratio[d] = d < L.hp.dim ? (L.hp.h[0] * L.hp.h[0]) / (L.hp.h[d] * L.hp.h[d]) : 1.0;
+  }
+  for (int i = 0; i < L.hp.n_t; ++i) q.tb[i] = L.hp.tau * L.hp.B_hat[i * L.hp.n_t + i];
+  return launch_diag_apply(mg.precision, L.hp.dim, L.hp.k, L.hp.n_t, q, s);
+}
+
 // r = b - A x in one apply (residual mode: the init kernel writes b minus the
 // Dirichlet rows, the cell kernel subtracts).
 template <typename T>
 cudaError_t residual(MG& mg, int l, cudaStream_t s, int trans) {
   MGLevel& L = mg.lv[l];
   if (L.use_diag) {
-    // the level operator couples no two rows (block Jacobi): the diagonal
-    // apply with per-row weights G_mu[alpha][alpha] (Psi_mu(xi_s) for samples)
-    McParams q;
-    std::memset(&q, 0, sizeof(q));
-    q.u_hi = -1;                       // every unit in one launch
-    q.bd_zero = 1;                     // x = b on the boundary (start, Vanka and transfers keep it)
-    q.n_prob = 1;
-    McProblem& P = q.pr[0];
-    P.x = L.d_x;
-    P.y = L.d_r;
-    P.b = L.d_b;
-    P.ctab = static_cast<const double*>(L.d_ctab);
-    P.wgt = mg.d_wgt;
-    P.amq = trans ? L.d_amqT : L.d_amq;
-    P.n_x = L.hp.n_x;
-    P.unit0 = 0;
-    P.n_cells = (int)L.hp.n_cells;
-    P.S = L.hp.n_xi;
-    P.ts = L.mc_ts;
-    P.tiles = (P.S + P.ts - 1) / P.ts;
-    for (int d = 0; d < 3; ++d) {
-      P.nn[d] = L.hp.nn[d];
-      P.cells[d] = L.hp.cells[d];
-      P.ratio[d] = d < L.hp.dim ? (L.hp.h[0] * L.hp.h[0]) / (L.hp.h[d] * L.hp.h[d]) : 0.0;
-    }
-    P.aniso = 0;
-    for (int d = 1; d < L.hp.dim; ++d) P.aniso |= L.hp.h[d] != L.hp.h[0];
-    q.n_terms = L.hp.n_terms;
-    q.chunk = L.mc_chunk;
-    q.mode = kApplyResidual;
-    q.mass_only = 0;
-    q.units = (long long)P.tiles * P.n_cells;
-    for (int i = 0; i < L.hp.n_t; ++i) q.tb[i] = L.hp.tau * L.hp.B_hat[i * L.hp.n_t + i];
-    return launch_mc_apply(mg.precision, L.hp.dim, L.hp.k, L.hp.n_t, q, L.mc_grid, L.mc_threads, L.mc_smem, s);
+    // the level operator couples no two rows (block Jacobi): the row-diagonal
+    // apply with the weights G_mu[alpha][alpha] (Psi_mu(xi_s) for samples).
+    // x = b on the boundary, as on every level, so the Dirichlet rows are 0.
+    const int V = L.hp.n_xi * L.hp.n_t;
+    launch_vec_start<T>(static_cast<const T*>(L.d_b), static_cast<const T*>(L.d_x), static_cast<T*>(L.d_r), nullptr, 4,
+                        V, L.hp.n_x, L.hp.nn, L.hp.dim, s);
+    return diag_residual(mg, L, s, trans);
   }
   ApplyParams p;
   fill_apply_params(L.hp, L.ls, L.d_ctab, L.d_grow, L.d_gcol, L.d_gterm, L.d_gval, L.d_perm, L.d_x, L.d_r, trans, p);
   p.b = L.d_b;
   p.mode = kApplyResidual;
   return launch_apply(L.hp, L.ls, p, s);
-}
-
-// The initial iterate (x = b on Dirichlet dofs, 0 inside) and its residual
-// (r = b inside, 0 on Dirichlet dofs) in one pass, without an apply.
-// Tile (rows) and chunk (cells) of a level's diagonal apply: the largest
-// chunk <= max_chunk within 100 KB of shared memory; the grid covers the units.
-sg_status level_diag_shape(MGLevel& L, int ts, int max_chunk, int vb) {
-  L.mc_ts = std::max(1, std::min(ts, L.hp.n_xi));
-  L.mc_chunk = 0;
-  for (int c = 1; c <= max_chunk; ++c)
-    if (mc_smem_bytes(L.hp.dim, L.hp.k, L.hp.n_t, L.mc_ts, L.hp.n_terms, c, vb) <= 100 * 1024) L.mc_chunk = c;
-  if (L.mc_chunk == 0) return SG_ERR_UNSUPPORTED;
-  L.mc_smem = mc_smem_bytes(L.hp.dim, L.hp.k, L.hp.n_t, L.mc_ts, L.hp.n_terms, L.mc_chunk, vb);
-  const long long units = (long long)((L.hp.n_xi + L.mc_ts - 1) / L.mc_ts) * L.hp.n_cells;
-  L.mc_grid = (int)std::max<long long>(1, std::min<long long>(units / std::max(1, L.mc_chunk), sg::sm_count() * 4));
-  return SG_OK;
 }
 
 // Shared memory of a Vanka chunk: r and the corrections of the tile's slots,
@@ -1175,49 +1154,31 @@ static float time_candidate(F&& launch, cudaStream_t s, cudaEvent_t a, cudaEvent
   return ms / 3.0f;
 }
 
-// Picks, for every smoothed level of at least 256 cells, the faster residual
-// apply on the level's own buffers: the diagonal apply over (rows per tile in
-// {8, 32, all} x at most 8 or 2 cells per chunk) or, where it applies, the SG
+// The residual apply of the smoothed levels.  The row-diagonal apply wins
+// wherever its values fit the registers with warps to spare (V-cycle with it
+// and with the SG cell kernel on every level, ms: 32^3 Q2 FP32 1.40 / 2.11,
+// FP64 17.1 / 17.7; 64^2 Q2 FP32 0.201 / 0.279, FP64 0.84 / 0.89; 64^2 Q3 dG(3)
+// FP32 0.70 / 0.73), but not for FP64 Q3 (254 registers; 8.60 / 8.22): those
+// levels of at least 256 cells are timed on their own buffers, against the SG
 // cell kernel over (cells per chunk x 256 / 512 threads), then the staggered
-// first chunk of the best cell-kernel shape.  Smaller levels keep the SG cell
-// kernel where it applies.
+// first chunk of its best shape.
 static cudaError_t tune_level_applies(MG& mg) {
-  const size_t vb = mg.precision == kPrecF32 ? 4 : 8;
+  if (mg.precision == kPrecF32 || mg.lv[0].hp.k < 3) return cudaSuccess;
+  const size_t vb = sizeof(double);
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   for (size_t l = 0; l < mg.lv.size() && e == cudaSuccess; ++l) {
     MGLevel& L = mg.lv[l];
     if (L.coarsest || L.hp.n_cells < 256) continue;
-    auto res = [&]() {
-      return mg.precision == kPrecF32 ? residual<float>(mg, (int)l, mg.stream, 0)
-                                      : residual<double>(mg, (int)l, mg.stream, 0);
-    };
+    auto res = [&]() { return residual<double>(mg, (int)l, mg.stream, 0); };
     const long long n = (long long)L.hp.n_xi * L.hp.n_t * L.hp.n_x;
     if ((e = cudaMemsetAsync(L.d_x, 0, n * vb, mg.stream)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(L.d_b, 0, n * vb, mg.stream)) != cudaSuccess) break;
-    std::vector<int> tss;
-    for (int t : {8, 32, L.hp.n_xi})
-      if (t <= L.hp.n_xi && std::find(tss.begin(), tss.end(), t) == tss.end()) tss.push_back(t);
-    int best_ts = L.mc_ts, best_c = 8;
-    float best_ms = 1e30f;
+    L.use_diag = true;
+    float best_ms = time_candidate(res, mg.stream, a, b, e);
     bool best_diag = true;
     LaunchShape best_ls = L.ls;
-    L.use_diag = true;
-    for (int ts : tss) {
-      for (int cmax : {8, 2}) {
-        if (e != cudaSuccess) break;
-        if (level_diag_shape(L, ts, cmax, (int)vb) != SG_OK) continue;
-        if (L.mc_chunk != cmax && cmax != 8) continue;           // the same shape as a larger cap
-        const float ms = time_candidate(res, mg.stream, a, b, e);
-        if (e == cudaSuccess && ms < best_ms) {
-          best_ms = ms;
-          best_ts = ts;
-          best_c = L.mc_chunk;
-        }
-      }
-    }
-    level_diag_shape(L, best_ts, best_c, (int)vb);
     if (L.chunk_ok) {
       // the SG cell kernel over (cells per chunk x threads)
       int dev = 0, optin = 0;
@@ -1361,14 +1322,15 @@ void mg_free(MG& mg) {
   cudaFree(mg.d_cls);
   cudaFree(mg.d_blk_cls);
   cudaFree(mg.d_blk_alpha);
-  cudaFree(mg.d_wgt);
+  cudaFree(mg.d_wused);
   cudaFree(mg.d_status);
-  mg.d_wgt = nullptr;
+  mg.d_wused = nullptr;
+  mg.used.clear();
   mg.d_status = nullptr;
   mg.d_blk_cls = mg.d_blk_alpha = nullptr;
   for (MGLevel& L : mg.lv) {
     cudaFree(L.d_ctab); cudaFree(L.d_grow); cudaFree(L.d_gcol); cudaFree(L.d_gterm); cudaFree(L.d_gval);
-    cudaFree(L.d_perm); cudaFree(L.d_inv); cudaFree(L.d_inner); cudaFree(L.d_amq); cudaFree(L.d_amqT);
+    cudaFree(L.d_perm); cudaFree(L.d_inv); cudaFree(L.d_inner); cudaFree(L.d_coef);
     cudaFree(L.d_x); cudaFree(L.d_b); cudaFree(L.d_r); cudaFree(L.d_t1); cudaFree(L.d_t2);
     for (int d = 0; d < 3; ++d) {
       cudaFree(L.d_pidx[d]); cudaFree(L.d_pwl[d]);
@@ -1468,6 +1430,22 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
     }
   mg.lv.resize(hps.size());
   cudaError_t e = cudaSuccess;
+  {
+    // per-row weights of the row-diagonal apply, G_mu[alpha][alpha], of the terms any row uses
+    for (int t = 0; t < fine.n_terms; ++t)
+      for (int a = 0; a < fine.n_xi; ++a)
+        if (drow[a][t] != 0.0) {
+          mg.used.push_back(t);
+          break;
+        }
+    std::vector<double> w;
+    for (int a = 0; a < fine.n_xi; ++a)
+      for (int t : mg.used) w.push_back(drow[a][t]);
+    if ((e = upload_values(&mg.d_wused, w, precision)) != cudaSuccess) {
+      msg = std::string("multigrid set-up: ") + cudaGetErrorString(e);
+      return e == cudaErrorMemoryAllocation ? SG_ERR_OOM : SG_ERR_CUDA;
+    }
+  }
   for (size_t l = 0; l < hps.size(); ++l) {
     MGLevel& L = mg.lv[l];
     L.hp = std::move(hps[l]);
@@ -1478,23 +1456,16 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
     L.coarsest = l + 1 == mg.lv.size();
     {
       // the level residual is the diagonal apply: time-mass tables of A_t and A_t^T
-      std::vector<double> amq, amqT, At((size_t)L.hp.n_t * L.hp.n_t);
+      std::vector<double> At((size_t)L.hp.n_t * L.hp.n_t);
       for (int i = 0; i < L.hp.n_t; ++i)
         for (int j = 0; j < L.hp.n_t; ++j) At[(size_t)i * L.hp.n_t + j] = L.hp.A_hat[(size_t)j * L.hp.n_t + i];
-      mc_amq(L.hp, L.hp.A_hat, amq);
-      mc_amq(L.hp, At, amqT);
-      if ((e = upload_vec(&L.d_amq, amq)) != cudaSuccess) break;
-      if ((e = upload_vec(&L.d_amqT, amqT)) != cudaSuccess) break;
-      if ((e = prepare_mc_kernel(precision, L.hp.dim, L.hp.k, L.hp.n_t)) != cudaSuccess) break;
-      if (level_diag_shape(L, mg.mc ? mg.mc_ts : std::min(L.hp.n_xi, 32), 8, precision == kPrecF32 ? 4 : 8) != SG_OK) {
-        msg = "multigrid level tile does not fit in shared memory";
-        return SG_ERR_UNSUPPORTED;
-      }
+      mc_amq(L.hp, L.hp.A_hat, L.amq[0]);
+      mc_amq(L.hp, At, L.amq[1]);
       // the SG cell kernel with the diagonal coupling table, where it applies
       std::string m2;
       L.chunk_ok = !mg.mc && plan_apply(L.hp, L.ls, m2) == SG_OK;
       if (L.chunk_ok && (e = prepare_apply_kernel(precision, L.hp.dim, L.hp.k, L.hp.n_t, L.ls.smem)) != cudaSuccess) break;
-      L.use_diag = !L.chunk_ok;
+      L.use_diag = true;
     }
     const int n = L.hp.k + 1;
     const int nkd = L.hp.dim == 2 ? n * n : n * n * n;
@@ -1526,6 +1497,9 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
     }
     // level apply tables (coefficient stays double; vectors use the MG precision)
     if ((e = upload_vec(reinterpret_cast<double**>(&L.d_ctab), L.hp.ctab)) != cudaSuccess) break;
+    if (!L.coarsest &&
+        (e = diag_coefficients(precision, L.hp, static_cast<const double*>(L.d_ctab), mg.used, &L.d_coef, 0)) != cudaSuccess)
+      break;
     if (!L.coarsest) {
       // Vanka patch inverses, assembled and factored on the device
       const int npp = vanka_row_pitch(L.np);
@@ -1603,13 +1577,6 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       if (e != cudaSuccess) break;
     }
   }
-  if (e == cudaSuccess && !mg.d_wgt) {
-    // per-row weights of the diagonal level apply: G_mu[alpha][alpha]
-    std::vector<double> wgt((size_t)fine.n_xi * fine.n_terms);
-    for (int a = 0; a < fine.n_xi; ++a)
-      for (int t = 0; t < fine.n_terms; ++t) wgt[(size_t)a * fine.n_terms + t] = drow[a][t];
-    e = upload_vec(&mg.d_wgt, wgt);
-  }
   if (e == cudaSuccess) e = upload_vec(&mg.d_cls, mg.cls);
   if (e == cudaSuccess) e = upload_vec(&mg.d_blk_cls, blk_cls);
   if (e == cudaSuccess) e = upload_vec(&mg.d_blk_alpha, blk_alpha);
@@ -1636,22 +1603,11 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
   return SG_OK;
 }
 
-sg_status mg_build_mc(const HostProblem& fine, int precision, int nu, double omega, const std::vector<double>& wgt,
-                      int ts, MG& mg, std::string& msg) {
-  if (ts < 1 || (size_t)fine.n_xi * fine.n_terms != wgt.size()) {
-    msg = "Monte-Carlo weights or tile size inconsistent";
-    return SG_ERR_ARG;
-  }
+sg_status mg_build_mc(const HostProblem& fine, int precision, int nu, double omega, MG& mg, std::string& msg) {
   mg.mc = true;
-  mg.mc_ts = std::min(ts, fine.n_xi);
   // Vanka tiles: a multiple of 8 samples whose patch data fit beside each other
   mg.vanka_tile = std::min(fine.n_xi, 64);
   if (mg.vanka_tile < fine.n_xi) mg.vanka_tile = 64;
-  cudaError_t e = upload_vec(&mg.d_wgt, wgt);
-  if (e != cudaSuccess) {
-    msg = cudaGetErrorString(e);
-    return SG_ERR_CUDA;
-  }
   return mg_build(fine, precision, nu, omega, mg, msg, true);
 }
 
