@@ -290,10 +290,10 @@ cudaError_t launch_apply(const HostProblem& hp, const LaunchShape& ls, const App
   const int op = prm.mode == kApplyResidual ? 1 : (prm.mode == kApplyAccumulate ? 3 : 2);
   if (hp.precision == kPrecF32)
     launch_vec_start<float>(static_cast<const float*>(prm.b), static_cast<const float*>(prm.x),
-                            static_cast<float*>(prm.y), nullptr, op, V, hp.n_x, hp.nn, hp.dim, stream);
+                            static_cast<float*>(prm.y), op, V, hp.n_x, hp.nn, hp.dim, stream);
   else
     launch_vec_start<double>(static_cast<const double*>(prm.b), static_cast<const double*>(prm.x),
-                             static_cast<double*>(prm.y), nullptr, op, V, hp.n_x, hp.nn, hp.dim, stream);
+                             static_cast<double*>(prm.y), op, V, hp.n_x, hp.nn, hp.dim, stream);
   void* f = select_kernel(hp.precision, hp.dim, hp.k, hp.n_t);
   if (!f) return cudaErrorInvalidValue;
   void* args[] = {const_cast<ApplyParams*>(&prm)};

@@ -247,20 +247,17 @@ struct MGLevel {
   void* d_x = nullptr;       // level vectors (N_xi * N_t * n_x values of the MG precision)
   void* d_b = nullptr;
   void* d_r = nullptr;
-  // transfer to and from the next coarser level, per direction d: the
-  // interpolation lists (fine node <- coarse nodes) and the restriction lists
-  // (coarse node <- fine nodes), padded to pmax / rmax entries per output
-  // (weight 0) and stored entry-major, [entry][output]; weights in the MG
-  // precision;
-  // d_t1 / d_t2 hold the intermediate arrays of the separable passes
-  int* d_pidx[3] = {nullptr, nullptr, nullptr};
-  void* d_pwl[3] = {nullptr, nullptr, nullptr};
-  int* d_ridx[3] = {nullptr, nullptr, nullptr};
-  void* d_rw[3] = {nullptr, nullptr, nullptr};
-  int pmax[3] = {0, 0, 0};    // entries per output of the padded lists
-  int rmax[3] = {0, 0, 0};
-  void* d_t1 = nullptr;
-  void* d_t2 = nullptr;
+  // transfers to (down) and from (up) the next coarser level: per direction
+  // the 1D lists, padded to `width` entries per output (weight 0) and stored
+  // entry-major, [entry][output], weights in the MG precision; `tile` output
+  // rows per block and the input rows of every tile
+  struct Transfer {
+    int* idx[3] = {nullptr, nullptr, nullptr};
+    void* w[3] = {nullptr, nullptr, nullptr};
+    int* range = nullptr;
+    int width = 0, tile = 0, max_rows = 0;
+    size_t smem = 0;
+  } down, up;
 };
 
 // Coarsening stops at the first level with at most this many interior

@@ -276,11 +276,11 @@ cudaError_t launch_mc_apply(int precision, int dim, int k, int n_t, const McPara
     if (precision == kPrecF32) {
       const float* b = static_cast<const float*>(P.b);
       launch_vec_start<float>(b ? b + off : nullptr, static_cast<const float*>(P.x) + off,
-                              static_cast<float*>(P.y) + off, nullptr, op, V, P.n_x, P.nn, dim, s);
+                              static_cast<float*>(P.y) + off, op, V, P.n_x, P.nn, dim, s);
     } else {
       const double* b = static_cast<const double*>(P.b);
       launch_vec_start<double>(b ? b + off : nullptr, static_cast<const double*>(P.x) + off,
-                               static_cast<double*>(P.y) + off, nullptr, op, V, P.n_x, P.nn, dim, s);
+                               static_cast<double*>(P.y) + off, op, V, P.n_x, P.nn, dim, s);
     }
   }
   cudaError_t e = cudaGetLastError();

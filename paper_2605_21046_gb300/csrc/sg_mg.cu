@@ -42,23 +42,6 @@ cudaError_t prepare_apply_kernel(int precision, int dim, int k, int n_t, size_t 
 namespace {
 
 // ------------------------------------------------------------------ kernels
-// Vector-wise kernels run on a 2D grid: blockIdx.y is the vector, the node
-// index within it stays 32-bit (no 64-bit division per element).
-inline dim3 vec_grid(long long n_x, int V) {
-  return dim3((unsigned)std::max<long long>(1, std::min<long long>((n_x + 255) / 256, 1024)), (unsigned)V);
-}
-
-template <typename T>
-__global__ void mg_init_x(const T* __restrict__ b, T* __restrict__ x, int n_x, int nnx, int nny, int nnz, int dim) {
-  const long long off = (long long)blockIdx.y * n_x;
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n_x; m += gridDim.x * blockDim.x) {
-    const int ix = m % nnx, rr = m / nnx, iy = rr % nny, iz = rr / nny;
-    bool bd = ix == 0 || ix == nnx - 1 || iy == 0 || iy == nny - 1;
-    if (dim == 3) bd = bd || iz == 0 || iz == nnz - 1;
-    x[off + m] = bd ? b[off + m] : T(0);
-  }
-}
-
 template <typename S, typename D>
 __global__ void mg_convert(const S* __restrict__ a, D* __restrict__ b, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -456,59 +439,152 @@ __global__ void __launch_bounds__(256, 2) mg_vanka(const VankaParams<T> p) {
   cp_async_wait_all();
 }
 
-// One pass of a separable grid transfer: along one axis of a structured
-// array [VA][nin][B] -> [VA][nout][B],
-//     out[va][jo][b] (+)= sum_k w[k][jo] in[va][idx[k][jo]][b],  k < W,
-// with the 1D restriction lists (coarse node <- fine nodes) or the 1D
-// interpolation lists (fine node <- coarse nodes) padded to W entries per
-// output (weight 0, index of the output's first entry) and stored entry-major,
-// so the lanes of a warp (consecutive outputs in the x pass, one output in the
-// others) read them coalesced or broadcast from L1.  Restriction P^T and
-// prolongation P are d such passes (x, y, z resp. z, y, x), which read every
-// value a few times instead of (k+1)^d-fold per output.  Each thread walks the
-// flat output index with a fixed stride, carrying (va, jo, b) along instead
-// of dividing for every element.
+// Grid transfers, one launch each: the d separable 1D passes of a tile of one
+// plane of output nodes, in shared memory.  A block takes one vector, one
+// plane along z (3D) and a tile of rows along y: it combines the planes of its
+// z list while loading, then does the x and y passes (restriction) or the y
+// and x passes (interpolation) between two shared arrays, so the intermediate
+// arrays never reach memory.  Bound by L2 and HBM traffic: a fine plane is
+// read for every coarse plane that lists it (2.5 times on average for Q2,
+// mostly from L2).  The 1D lists (coarse node <- fine nodes, fine node <-
+// coarse nodes) are padded to W entries per output (weight 0, an index the
+// output's neighbours use) and stored entry-major; a thread keeps one output
+// column, with its list in registers, and walks the rows.
+//
+// The vectors that the next kernels reduce into are preset here, where their
+// nodes are written anyway: restriction also writes the coarse level's start
+// (x = 0, r = b; b vanishes on the boundary), interpolation r = b inside and 0
+// on the boundary for the residual that follows.
 constexpr int kAxisMax = 16;  // entries of one output of a 1D transfer list, at most (4k + 1 for k <= 3)
+constexpr int kTransferThreads = 256;
 
+template <typename T>
+struct TransferParams {
+  const T* in;              // restriction: fine residual; interpolation: coarse correction
+  const T* b;               // interpolation: fine right-hand side
+  T *out, *x, *r;           // restriction: b, x, r of the coarse level; interpolation: fine x (out), r
+  const int* idx[3];
+  const T* w[3];
+  const int* range;         // first and number of input rows of every tile
+  long long n_in, n_out;    // nodes per vector
+  int ni[3], no[3];         // nodes per direction of the input and output grids
+  int tile, max_rows, z;    // output rows per tile, most input rows of one; 3D
+  int cb_in, cb_out;        // columns a pass takes at a time, of the input and output grids
+  long long lim_in, lim_out;   // values of the vectors (bounds checks)
+};
+
+// The input rows [lo, lo + cnt) of the tile, combined along z, into S0 (row pitch ni[0]).
 template <typename T, int W>
-__global__ void __launch_bounds__(256) mg_axis_gather(const T* __restrict__ in, T* __restrict__ out, long long VA,
-                                                      int nin, int nout, int B, const int* __restrict__ idx,
-                                                      const T* __restrict__ w, int accumulate) {
-  const long long total = VA * nout * B;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= total) return;
-  int b = (int)(e % B);
-  long long r = e / B;
-  int jo = (int)(r % nout);
-  long long va = r / nout;
-  const int db = (int)(stride % B);
-  const long long rs = stride / B;
-  const int djo = (int)(rs % nout);
-  const long long dva = rs / nout;
-  const long long row_in = (long long)nin * B;
-  for (; e < total; e += stride) {
-    const T* src = in + va * row_in + b;
-    T acc = T(0);
+__device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz, int lo, int cnt, T* S0) {
+  const long long v_in = (long long)blockIdx.x * p.n_in;
+  const T* src = p.in + v_in;
+  const int n = cnt * p.ni[0], off = lo * p.ni[0];
+  if (p.z) {
+    const int plane = p.ni[0] * p.ni[1];
+    const T* pl[W];
+    T wz[W];
+    int m = 0;
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-      const int si = __ldg(idx + k * nout + jo);
-      if (SG_IN(si, nin, 501)) acc += __ldg(w + k * nout + jo) * src[(long long)si * B];
+      const T wk = __ldg(p.w[2] + k * p.no[2] + jz);
+      wz[k] = wk;
+      pl[k] = src + (long long)__ldg(p.idx[2] + k * p.no[2] + jz) * plane + off;
+      if (wk != T(0)) m = k + 1;
     }
-    if (accumulate) out[e] += acc;
-    else out[e] = acc;
-    b += db;
-    jo += djo;
-    va += dva;
-    if (b >= B) {
-      b -= B;
-      ++jo;
+    for (int i = threadIdx.x; i < n; i += kTransferThreads) {
+      T s = T(0);
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (k < m && SG_IN(pl[k] - p.in + i, p.lim_in, 501)) s = fma(wz[k], __ldg(pl[k] + i), s);
+      S0[i] = s;
     }
-    if (jo >= nout) {
-      jo -= nout;
-      ++va;
+  } else {
+    for (int i = threadIdx.x; i < n; i += kTransferThreads)
+      if (SG_IN(v_in + off + i, p.lim_in, 501)) S0[i] = __ldg(src + off + i);
+  }
+}
+
+// One 1D pass along x or y of `rows` output rows: DIR 0 out[row][c] = sum_k w in[row][idx[c]],
+// DIR 1 out[row][c] = sum_k w in[idx[row0 + row] - lo][c]; put(row, column, value).
+template <typename T, int W, int DIR, class Put>
+__device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, int cb, int rows, const int* idx,
+                                              const T* w, int n_list, int row0, int lo, Put put) {
+  const int par = kTransferThreads / cb;                       // cb columns x par rows at a time
+  const int c0 = threadIdx.x % cb, r0 = threadIdx.x / cb;
+  if (r0 >= par) return;
+  for (int c = c0; c < cols; c += cb) {
+    if constexpr (DIR == 0) {
+      int at[W];
+      T wt[W];
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        at[k] = __ldg(idx + k * n_list + c);
+        wt[k] = __ldg(w + k * n_list + c);
+      }
+      for (int r = r0; r < rows; r += par) {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < W; ++k) s = fma(wt[k], in[r * pitch + at[k]], s);
+        put(r, c, s);
+      }
+    } else {
+      for (int r = r0; r < rows; r += par) {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          s = fma(__ldg(w + k * n_list + row0 + r), in[(__ldg(idx + k * n_list + row0 + r) - lo) * pitch + c], s);
+        put(r, c, s);
+      }
     }
   }
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(kTransferThreads) mg_restrict(const TransferParams<T> p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][fine x]
+  T* S1 = S0 + (size_t)p.max_rows * p.ni[0];                    // [max_rows][coarse x]
+  const int jz = blockIdx.y, j0 = blockIdx.z * p.tile, nj = min(p.tile, p.no[1] - j0);
+  const int lo = __ldg(p.range + 2 * blockIdx.z), cnt = __ldg(p.range + 2 * blockIdx.z + 1);
+  transfer_load<T, W>(p, jz, lo, cnt, S0);
+  __syncthreads();
+  const int ncx = p.no[0];
+  transfer_pass<T, W, 0>(S0, p.ni[0], ncx, p.cb_out, cnt, p.idx[0], p.w[0], ncx, 0, 0,
+                         [&](int r, int c, T v) { S1[r * ncx + c] = v; });
+  __syncthreads();
+  const long long o0 = (long long)blockIdx.x * p.n_out + ((long long)jz * p.no[1] + j0) * ncx;
+  transfer_pass<T, W, 1>(S1, ncx, ncx, p.cb_out, nj, p.idx[1], p.w[1], p.no[1], j0, lo, [&](int r, int c, T v) {
+    const long long o = o0 + (long long)r * ncx + c;
+    if (!SG_IN(o, p.lim_out, 502)) return;
+    p.out[o] = v;
+    p.x[o] = T(0);
+    p.r[o] = v;
+  });
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferParams<T> p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][coarse x]
+  T* S1 = S0 + (size_t)p.max_rows * p.ni[0];                    // [tile][coarse x]
+  const int jz = blockIdx.y, j0 = blockIdx.z * p.tile, nj = min(p.tile, p.no[1] - j0);
+  const int lo = __ldg(p.range + 2 * blockIdx.z), cnt = __ldg(p.range + 2 * blockIdx.z + 1);
+  transfer_load<T, W>(p, jz, lo, cnt, S0);
+  __syncthreads();
+  const int ncx = p.ni[0], nfx = p.no[0];
+  transfer_pass<T, W, 1>(S0, ncx, ncx, p.cb_in, nj, p.idx[1], p.w[1], p.no[1], j0, lo,
+                         [&](int r, int c, T v) { S1[r * ncx + c] = v; });
+  __syncthreads();
+  const long long o0 = (long long)blockIdx.x * p.n_out + ((long long)jz * p.no[1] + j0) * nfx;
+  const bool edge_z = p.z && (jz == 0 || jz == p.no[2] - 1);
+  transfer_pass<T, W, 0>(S1, ncx, nfx, p.cb_out, nj, p.idx[0], p.w[0], nfx, 0, 0, [&](int r, int c, T v) {
+    const long long o = o0 + (long long)r * nfx + c;
+    if (!SG_IN(o, p.lim_out, 503)) return;
+    const int jy = j0 + r;
+    const bool bd = edge_z || jy == 0 || jy == p.no[1] - 1 || c == 0 || c == nfx - 1;
+    p.out[o] += v;
+    p.r[o] = bd ? T(0) : p.b[o];
+  });
 }
 
 // Coarsest level: x[inner] = inv(C_class) b[inner] for every chaos mode
@@ -855,16 +931,17 @@ cudaError_t diag_residual(MG& mg, MGLevel& L, cudaStream_t s, int trans) {
 
 // r = b - A x in one apply (residual mode: the init kernel writes b minus the
 // Dirichlet rows, the cell kernel subtracts).
+// `preset`: r already holds b inside and 0 on the boundary.
 template <typename T>
-cudaError_t residual(MG& mg, int l, cudaStream_t s, int trans) {
+cudaError_t residual(MG& mg, int l, cudaStream_t s, int trans, bool preset) {
   MGLevel& L = mg.lv[l];
   if (L.use_diag) {
     // the level operator couples no two rows (block Jacobi): the row-diagonal
     // apply with the weights G_mu[alpha][alpha] (Psi_mu(xi_s) for samples).
     // x = b on the boundary, as on every level, so the Dirichlet rows are 0.
-    const int V = L.hp.n_xi * L.hp.n_t;
-    launch_vec_start<T>(static_cast<const T*>(L.d_b), static_cast<const T*>(L.d_x), static_cast<T*>(L.d_r), nullptr, 4,
-                        V, L.hp.n_x, L.hp.nn, L.hp.dim, s);
+    if (!preset)
+      launch_vec_start<T>(static_cast<const T*>(L.d_b), static_cast<const T*>(L.d_x), static_cast<T*>(L.d_r), 4,
+                          L.hp.n_xi * L.hp.n_t, L.hp.n_x, L.hp.nn, L.hp.dim, s);
     return diag_residual(mg, L, s, trans);
   }
   ApplyParams p;
@@ -1010,29 +1087,6 @@ bool vk_launch(MG& mg, MGLevel& L, cudaStream_t s) {
   return mg.precision == kPrecF32 ? vanka<float>(mg, L, s, 0) : vanka<double>(mg, L, s, 0);
 }
 
-template <typename T, int W>
-void axis_pass_w(const void* in, void* out, long long VA, int nin, int nout, int B, const int* idx, const void* w,
-                 int accumulate, cudaStream_t s) {
-  const long long total = VA * nout * B;
-  const int grid = (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, sg::sm_count() * 8));
-  mg_axis_gather<T, W><<<grid, 256, 0, s>>>(static_cast<const T*>(in), static_cast<T*>(out), VA, nin, nout, B, idx,
-                                            static_cast<const T*>(w), accumulate);
-}
-
-// one pass with lists padded to width (one of axis_width's values)
-template <typename T>
-void axis_pass(const void* in, void* out, long long VA, int nin, int nout, int B, const int* idx, const void* w,
-               int width, int accumulate, cudaStream_t s) {
-  switch (width) {
-    case 2: axis_pass_w<T, 2>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-    case 3: axis_pass_w<T, 3>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-    case 4: axis_pass_w<T, 4>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-    case 5: axis_pass_w<T, 5>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-    case 8: axis_pass_w<T, 8>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-    default: axis_pass_w<T, kAxisMax>(in, out, VA, nin, nout, B, idx, w, accumulate, s); break;
-  }
-}
-
 // the padded width of lists whose longest has n entries
 int axis_width(int n) {
   for (int w : {2, 3, 4, 5, 8})
@@ -1049,56 +1103,129 @@ void pad_lists(const std::vector<int>& ptr, const std::vector<int>& idx, const s
   for (int o = 0; o < n; ++o) {
     const int c = ptr[o + 1] - ptr[o];
     for (int k = 0; k < width; ++k) {
-      pidx[(size_t)k * n + o] = k < c ? idx[ptr[o] + k] : (c > 0 ? idx[ptr[o]] : 0);
+      pidx[(size_t)k * n + o] = k < c ? idx[ptr[o] + k] : (c > 0 ? idx[ptr[o]] : -1);
       pw[(size_t)k * n + o] = k < c ? wt[ptr[o] + k] : 0.0;
     }
   }
+  // outputs without entries (Dirichlet nodes) point where their neighbour does
+  for (int k = 0; k < width; ++k)
+    for (int pass = 0; pass < 2; ++pass)
+      for (int i = 1; i < n; ++i) {
+        const int o = pass ? n - 1 - i : i, nb = pass ? o + 1 : o - 1;
+        int& at = pidx[(size_t)k * n + o];
+        if (at < 0) at = pidx[(size_t)k * n + nb];
+      }
+  for (int& at : pidx) at = std::max(at, 0);
 }
 
-// x_fine += P e_coarse: interpolation along z (3D), y, then x
-template <typename T>
-bool prolong(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
-  const int nfx = F.hp.nn[0], nfy = F.hp.nn[1], nfz = F.hp.nn[2];
-  const int ncx = C.hp.nn[0], ncy = C.hp.nn[1], ncz = C.hp.nn[2];
-  auto pass = [&](const void* in, void* out, long long VA, int nin, int nout, int B, int d, int acc) {
-    axis_pass<T>(in, out, VA, nin, nout, B, F.d_pidx[d], F.d_pwl[d], F.pmax[d], acc, s);
-  };
-  if (F.hp.dim == 3) {
-    pass(C.d_x, F.d_t2, V, ncz, nfz, ncy * ncx, 2, 0);
-    pass(F.d_t2, F.d_t1, (long long)V * nfz, ncy, nfy, ncx, 1, 0);
-    pass(F.d_t1, F.d_x, (long long)V * nfz * nfy, ncx, nfx, 1, 0, 1);
-  } else {
-    pass(C.d_x, F.d_t1, V, ncy, nfy, ncx, 1, 0);
-    pass(F.d_t1, F.d_x, (long long)V * nfy, ncx, nfx, 1, 0, 1);
+// The tiles of `tile` outputs each of a padded list: first input and number of inputs, per tile.
+int tile_ranges(const std::vector<int>& pidx, int width, int n, int tile, std::vector<int>& range) {
+  int most = 0;
+  range.clear();
+  for (int o0 = 0; o0 < n; o0 += tile) {
+    int lo = pidx[o0], hi = lo;
+    for (int o = o0; o < std::min(n, o0 + tile); ++o)
+      for (int k = 0; k < width; ++k) {
+        lo = std::min(lo, pidx[(size_t)k * n + o]);
+        hi = std::max(hi, pidx[(size_t)k * n + o]);
+      }
+    range.push_back(lo);
+    range.push_back(hi - lo + 1);
+    most = std::max(most, hi - lo + 1);
   }
-  return cudaGetLastError() == cudaSuccess;
+  return most;
 }
 
-// b_coarse = P^T r_fine: restriction along x, y, then z (3D)
-template <typename T>
-void restrict_to(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
-  const int nfx = F.hp.nn[0], nfy = F.hp.nn[1], nfz = F.hp.nn[2];
-  const int ncx = C.hp.nn[0], ncy = C.hp.nn[1], ncz = C.hp.nn[2];
-  auto pass = [&](const void* in, void* out, long long VA, int nin, int nout, int B, int d) {
-    axis_pass<T>(in, out, VA, nin, nout, B, F.d_ridx[d], F.d_rw[d], F.rmax[d], 0, s);
-  };
-  if (F.hp.dim == 3) {
-    pass(F.d_r, F.d_t1, (long long)V * nfz * nfy, nfx, ncx, 1, 0);
-    pass(F.d_t1, F.d_t2, (long long)V * nfz, nfy, ncy, ncx, 1);
-    pass(F.d_t2, C.d_b, V, nfz, ncz, ncy * ncx, 2);
-  } else {
-    pass(F.d_r, F.d_t1, (long long)V * nfy, nfx, ncx, 1, 0);
-    pass(F.d_t1, C.d_b, V, nfy, ncy, ncx, 1);
+// Columns a pass takes at a time: as few parts of a row as keep three quarters
+// of the threads busy (129 nodes: 65 x 3 rows instead of 129 x 1).
+int column_block(int cols) {
+  int best = std::min(cols, kTransferThreads);
+  for (int m = 1; m <= 16; ++m) {
+    const int cb = std::min((cols + m - 1) / m, kTransferThreads);
+    const int busy = kTransferThreads / cb * cb, had = kTransferThreads / best * best;
+    if (busy >= 3 * kTransferThreads / 4) return cb;
+    if (busy > had) best = cb;
   }
+  return best;
+}
+
+template <typename T>
+void transfer_params(const MGLevel& I, const MGLevel& O, const MGLevel::Transfer& t, int V, TransferParams<T>& p) {
+  for (int d = 0; d < 3; ++d) {
+    p.idx[d] = t.idx[d];
+    p.w[d] = static_cast<const T*>(t.w[d]);
+    p.ni[d] = I.hp.nn[d];
+    p.no[d] = O.hp.nn[d];
+  }
+  p.range = t.range;
+  p.n_in = I.hp.n_x;
+  p.n_out = O.hp.n_x;
+  p.tile = t.tile;
+  p.max_rows = t.max_rows;
+  p.z = I.hp.dim == 3;
+  p.cb_in = column_block(p.ni[0]);
+  p.cb_out = column_block(p.no[0]);
+  p.lim_in = (long long)V * I.hp.n_x;
+  p.lim_out = (long long)V * O.hp.n_x;
+}
+
+// Bytes of shared memory of a transfer block: the input rows, and the rows
+// between its two passes (restriction: the input rows; interpolation: the tile).
+size_t transfer_smem(bool up, int max_rows, int tile, int nfx, int ncx, size_t vb) {
+  return vb * (up ? (size_t)max_rows * ncx + (size_t)tile * ncx : (size_t)max_rows * (nfx + ncx));
+}
+
+#define SG_TRANSFER_WIDTHS(CALL) \
+  switch (t.width) {             \
+    case 2: CALL(2); break;      \
+    case 3: CALL(3); break;      \
+    case 4: CALL(4); break;      \
+    case 5: CALL(5); break;      \
+    case 8: CALL(8); break;      \
+    default: CALL(kAxisMax); break; \
+  }
+
+// x_fine += P e_coarse; r_fine = b_fine inside, 0 on the boundary
+template <typename T>
+cudaError_t prolong(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
+  const MGLevel::Transfer& t = F.up;
+  TransferParams<T> p;
+  transfer_params(C, F, t, V, p);
+  p.in = static_cast<const T*>(C.d_x);
+  p.b = static_cast<const T*>(F.d_b);
+  p.out = static_cast<T*>(F.d_x);
+  p.x = nullptr;
+  p.r = static_cast<T*>(F.d_r);
+  const dim3 grid(V, p.z ? p.no[2] : 1, (p.no[1] + t.tile - 1) / t.tile);
+#define SG_CALL(W) mg_prolong<T, W><<<grid, kTransferThreads, t.smem, s>>>(p)
+  SG_TRANSFER_WIDTHS(SG_CALL)
+#undef SG_CALL
+  return cudaGetLastError();
+}
+
+// b_coarse = P^T r_fine; x_coarse = 0, r_coarse = b_coarse
+template <typename T>
+cudaError_t restrict_to(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
+  const MGLevel::Transfer& t = F.down;
+  TransferParams<T> p;
+  transfer_params(F, C, t, V, p);
+  p.in = static_cast<const T*>(F.d_r);
+  p.b = nullptr;
+  p.out = static_cast<T*>(C.d_b);
+  p.x = static_cast<T*>(C.d_x);
+  p.r = static_cast<T*>(C.d_r);
+  const dim3 grid(V, p.z ? p.no[2] : 1, (p.no[1] + t.tile - 1) / t.tile);
+#define SG_CALL(W) mg_restrict<T, W><<<grid, kTransferThreads, t.smem, s>>>(p)
+  SG_TRANSFER_WIDTHS(SG_CALL)
+#undef SG_CALL
+  return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t issue_vcycle(MG& mg, int l, cudaStream_t s, int trans) {
   MGLevel& L = mg.lv[l];
   const int V = L.hp.n_xi * L.hp.n_t;
-  if (L.coarsest) {
-    mg_init_x<T><<<vec_grid(L.hp.n_x, V), 256, 0, s>>>(static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x),
-                                                      (int)L.hp.n_x, L.hp.nn[0], L.hp.nn[1], L.hp.nn[2], L.hp.dim);
+  if (L.coarsest) {   // x holds the boundary values and 0 inside (restriction, or the start of a one-level hierarchy)
     const size_t smem = (size_t)L.n_int * sizeof(T);
     const int gx = trans ? (L.n_int + 255) / 256 : (L.n_int + 7) / 8;   // rows: a warp each (8 a block)
     mg_coarse<T><<<dim3(gx, L.hp.n_xi), 256, smem, s>>>(static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x),
@@ -1108,25 +1235,25 @@ cudaError_t issue_vcycle(MG& mg, int l, cudaStream_t s, int trans) {
     return cudaGetLastError();
   }
   cudaError_t e;
-  // the start: x = the boundary values of b and 0 inside; the first sweep's
-  // residual b - A x is b on the interior, where the sweep reads it
-  launch_vec_start<T>(nullptr, static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x), nullptr, 2, V, L.hp.n_x,
-                      L.hp.nn, L.hp.dim, s);
+  // the level arrives started: x = the boundary values of b and 0 inside,
+  // r = b inside and 0 on the boundary.  The first sweep's residual b - A x is
+  // b on the interior, where the sweep reads it; r is then the preset of the
+  // residual that follows.
   for (int it = 0; it < mg.nu; ++it) {
-    if (it > 0 && (e = residual<T>(mg, l, s, trans)) != cudaSuccess) return e;
+    if (it > 0 && (e = residual<T>(mg, l, s, trans, it == 1)) != cudaSuccess) return e;
     L.vanka_r = it == 0 ? L.d_b : nullptr;
     const bool ok = vanka<T>(mg, L, s, trans);
     L.vanka_r = nullptr;
     if (!ok) return cudaErrorInvalidValue;
   }
-  if ((e = residual<T>(mg, l, s, trans)) != cudaSuccess) return e;
+  if ((e = residual<T>(mg, l, s, trans, mg.nu == 1)) != cudaSuccess) return e;
   MGLevel& C = mg.lv[l + 1];
   if (C.hp.n_xi * C.hp.n_t != V) return cudaErrorInvalidValue;   // level buffers hold V vectors
-  restrict_to<T>(L, C, V, s);
+  if ((e = restrict_to<T>(L, C, V, s)) != cudaSuccess) return e;
   if ((e = issue_vcycle<T>(mg, l + 1, s, trans)) != cudaSuccess) return e;
-  if (!prolong<T>(L, C, V, s)) return cudaErrorInvalidValue;
+  if ((e = prolong<T>(L, C, V, s)) != cudaSuccess) return e;
   for (int it = 0; it < mg.nu; ++it) {
-    if ((e = residual<T>(mg, l, s, trans)) != cudaSuccess) return e;
+    if ((e = residual<T>(mg, l, s, trans, it == 0)) != cudaSuccess) return e;
     if (!vanka<T>(mg, L, s, trans)) return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -1171,7 +1298,7 @@ static cudaError_t tune_level_applies(MG& mg) {
   for (size_t l = 0; l < mg.lv.size() && e == cudaSuccess; ++l) {
     MGLevel& L = mg.lv[l];
     if (L.coarsest || L.hp.n_cells < 256) continue;
-    auto res = [&]() { return residual<double>(mg, (int)l, mg.stream, 0); };
+    auto res = [&]() { return residual<double>(mg, (int)l, mg.stream, 0, false); };
     const long long n = (long long)L.hp.n_xi * L.hp.n_t * L.hp.n_x;
     if ((e = cudaMemsetAsync(L.d_x, 0, n * vb, mg.stream)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(L.d_b, 0, n * vb, mg.stream)) != cudaSuccess) break;
@@ -1331,15 +1458,86 @@ void mg_free(MG& mg) {
   for (MGLevel& L : mg.lv) {
     cudaFree(L.d_ctab); cudaFree(L.d_grow); cudaFree(L.d_gcol); cudaFree(L.d_gterm); cudaFree(L.d_gval);
     cudaFree(L.d_perm); cudaFree(L.d_inv); cudaFree(L.d_inner); cudaFree(L.d_coef);
-    cudaFree(L.d_x); cudaFree(L.d_b); cudaFree(L.d_r); cudaFree(L.d_t1); cudaFree(L.d_t2);
-    for (int d = 0; d < 3; ++d) {
-      cudaFree(L.d_pidx[d]); cudaFree(L.d_pwl[d]);
-      cudaFree(L.d_ridx[d]); cudaFree(L.d_rw[d]);
+    cudaFree(L.d_x); cudaFree(L.d_b); cudaFree(L.d_r);
+    for (MGLevel::Transfer* t : {&L.down, &L.up}) {
+      for (int d = 0; d < 3; ++d) {
+        cudaFree(t->idx[d]);
+        cudaFree(t->w[d]);
+      }
+      cudaFree(t->range);
     }
   }
   mg.lv.clear();
   mg.stream = nullptr;
   mg.d_cls = nullptr;
+}
+
+// Lets the transfer kernels use more than 48 KB of shared memory (rows of
+// more than about 1000 nodes).
+template <typename T, int W>
+static cudaError_t prepare_transfers_w(int optin) {
+  cudaError_t e = cudaFuncSetAttribute(&mg_restrict<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  return e == cudaSuccess ? cudaFuncSetAttribute(&mg_prolong<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)
+                          : e;
+}
+template <typename T>
+static cudaError_t prepare_transfers_t() {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaError_t e = cudaSuccess;
+  for (auto f : {&prepare_transfers_w<T, 2>, &prepare_transfers_w<T, 3>, &prepare_transfers_w<T, 4>,
+                 &prepare_transfers_w<T, 5>, &prepare_transfers_w<T, 8>, &prepare_transfers_w<T, kAxisMax>})
+    if (e == cudaSuccess) e = f(optin);
+  return e;
+}
+static cudaError_t prepare_transfers(size_t vb) {
+  return vb == 4 ? prepare_transfers_t<float>() : prepare_transfers_t<double>();
+}
+
+// The transfers between a level F and the next coarser one: the 1D lists of
+// every direction padded to one width, and the tiles of the plane kernels.
+// Rows per tile: halved from the whole plane until a block's rows fit in 48 KB
+// of shared memory and the blocks cover the GPU four times, or 4 rows are left
+// (64^2 Q2, 70 vectors: 8 rows, 630 blocks; 32^3 Q2: whole planes of 65 rows).
+static cudaError_t build_transfers(MGLevel& F, const MGLevel& C, size_t vb) {
+  std::vector<int> ptr[2][3], idx[2][3];
+  std::vector<double> w[2][3];
+  int longest[2] = {0, 0};
+  for (int d = 0; d < F.hp.dim; ++d) {
+    transfer_1d(F.hp, C.hp, d, ptr[1][d], idx[1][d], w[1][d], ptr[0][d], idx[0][d], w[0][d]);
+    for (int u = 0; u < 2; ++u)
+      for (size_t i = 0; i + 1 < ptr[u][d].size(); ++i) longest[u] = std::max(longest[u], ptr[u][d][i + 1] - ptr[u][d][i]);
+  }
+  cudaError_t e = cudaSuccess;
+  const int precision = vb == 4 ? kPrecF32 : SG_PREC_FP64;
+  for (int u = 0; u < 2; ++u) {
+    MGLevel::Transfer& t = u ? F.up : F.down;
+    if (longest[u] > kAxisMax) return cudaErrorInvalidValue;
+    t.width = axis_width(longest[u]);
+    std::vector<int> pi, py;
+    std::vector<double> pw;
+    for (int d = 0; d < F.hp.dim; ++d) {
+      pad_lists(ptr[u][d], idx[u][d], w[u][d], t.width, pi, pw);
+      if (d == 1) py = pi;
+      if ((e = upload_vec(&t.idx[d], pi)) != cudaSuccess) return e;
+      if ((e = upload_values(&t.w[d], pw, precision)) != cudaSuccess) return e;
+    }
+    const HostProblem& out = u ? F.hp : C.hp;
+    const long long planes = (long long)F.hp.n_xi * F.hp.n_t * (F.hp.dim == 3 ? out.nn[2] : 1);
+    std::vector<int> range;
+    t.tile = out.nn[1];
+    while (true) {
+      t.max_rows = tile_ranges(py, t.width, out.nn[1], t.tile, range);
+      t.smem = transfer_smem(u == 1, t.max_rows, t.tile, F.hp.nn[0], C.hp.nn[0], vb);
+      const long long blocks = planes * ((out.nn[1] + t.tile - 1) / t.tile);
+      if (t.tile == 1 || (t.smem <= 48 * 1024 && (blocks >= 4 * sg::sm_count() || t.tile <= 4))) break;
+      t.tile = (t.tile + 1) / 2;
+    }
+    if (t.smem > 48 * 1024 && (e = prepare_transfers(vb)) != cudaSuccess) return e;
+    if ((e = upload_vec(&t.range, range)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega, MG& mg, std::string& msg,
@@ -1543,38 +1741,7 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
     if ((e = cudaMalloc(&L.d_r, bytes)) != cudaSuccess) break;
     if (l > 0) {
       MGLevel& F = mg.lv[l - 1];
-      for (int d = 0; d < F.hp.dim; ++d) {
-        std::vector<int> pptr, pidx, rptr, ridx;
-        std::vector<double> pwl, rw;
-        transfer_1d(F.hp, L.hp, d, pptr, pidx, pwl, rptr, ridx, rw);
-        int pm = 0, rm = 0;
-        for (size_t i = 0; i + 1 < pptr.size(); ++i) pm = std::max(pm, pptr[i + 1] - pptr[i]);
-        for (size_t j = 0; j + 1 < rptr.size(); ++j) rm = std::max(rm, rptr[j + 1] - rptr[j]);
-        if (pm > kAxisMax || rm > kAxisMax) {
-          e = cudaErrorInvalidValue;
-          break;
-        }
-        F.pmax[d] = axis_width(pm);
-        F.rmax[d] = axis_width(rm);
-        std::vector<int> pi, ri;
-        std::vector<double> pwv, rwv;
-        pad_lists(pptr, pidx, pwl, F.pmax[d], pi, pwv);
-        pad_lists(rptr, ridx, rw, F.rmax[d], ri, rwv);
-        if ((e = upload_vec(&F.d_pidx[d], pi)) != cudaSuccess) break;
-        if ((e = upload_values(&F.d_pwl[d], pwv, precision)) != cudaSuccess) break;
-        if ((e = upload_vec(&F.d_ridx[d], ri)) != cudaSuccess) break;
-        if ((e = upload_values(&F.d_rw[d], rwv, precision)) != cudaSuccess) break;
-      }
-      if (e != cudaSuccess) break;
-      // intermediate arrays of the separable transfers between F and this level
-      {
-        const long long V = (long long)F.hp.n_xi * F.hp.n_t;
-        const long long t1 = V * F.hp.nn[2] * F.hp.nn[1] * L.hp.nn[0];
-        const long long t2 = F.hp.dim == 3 ? V * F.hp.nn[2] * L.hp.nn[1] * L.hp.nn[0] : 1;
-        if ((e = cudaMalloc(&F.d_t1, t1 * vb)) != cudaSuccess) break;
-        if ((e = cudaMalloc(&F.d_t2, t2 * vb)) != cudaSuccess) break;
-      }
-      if (e != cudaSuccess) break;
+      if ((e = build_transfers(F, L, vb)) != cudaSuccess) break;
     }
   }
   if (e == cudaSuccess) e = upload_vec(&mg.d_cls, mg.cls);
@@ -1745,29 +1912,38 @@ sg_status mg_patch_inverse(const MG& mg, int level, int alpha, long long cell, d
   return SG_OK;
 }
 
-cudaError_t mg_issue(MG& mg, const double* r, double* z, cudaStream_t stream, int trans) {
-  MGLevel& L0 = mg.lv[0];
-  const long long n = (long long)L0.hp.n_xi * L0.hp.n_t * L0.hp.n_x;
-  const bool f32 = mg.precision == kPrecF32;
-  const int t = trans ? 1 : 0;
-  cudaError_t e;
-  if (f32)
-    mg_convert<double, float><<<grid_for(n, 256), 256, 0, stream>>>(r, static_cast<float*>(L0.d_b), n);
+// b = r in the MG precision, and the start of the finest level (x, r)
+static cudaError_t mg_enter(MG& mg, const double* r, cudaStream_t s) {
+  MGLevel& L = mg.lv[0];
+  const int V = L.hp.n_xi * L.hp.n_t;
+  if (mg.precision == kPrecF32)
+    launch_vec_enter<float>(r, static_cast<float*>(L.d_b), static_cast<float*>(L.d_x), static_cast<float*>(L.d_r), V,
+                            L.hp.n_x, L.hp.nn, L.hp.dim, s);
   else
-    mg_convert<double, double><<<grid_for(n, 256), 256, 0, stream>>>(r, static_cast<double*>(L0.d_b), n);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = f32 ? issue_vcycle<float>(mg, 0, stream, t) : issue_vcycle<double>(mg, 0, stream, t)) != cudaSuccess)
-    return e;
-  if (f32)
-    mg_convert<float, double><<<grid_for(n, 256), 256, 0, stream>>>(static_cast<const float*>(L0.d_x), z, n);
-  else
-    mg_convert<double, double><<<grid_for(n, 256), 256, 0, stream>>>(static_cast<const double*>(L0.d_x), z, n);
+    launch_vec_enter<double>(r, static_cast<double*>(L.d_b), static_cast<double*>(L.d_x), static_cast<double*>(L.d_r), V,
+                             L.hp.n_x, L.hp.nn, L.hp.dim, s);
   return cudaGetLastError();
 }
 
+static cudaError_t mg_leave(MG& mg, double* z, cudaStream_t s) {
+  MGLevel& L = mg.lv[0];
+  const long long n = (long long)L.hp.n_xi * L.hp.n_t * L.hp.n_x;
+  if (mg.precision == kPrecF32)
+    mg_convert<float, double><<<grid_for(n, 256), 256, 0, s>>>(static_cast<const float*>(L.d_x), z, n);
+  else
+    mg_convert<double, double><<<grid_for(n, 256), 256, 0, s>>>(static_cast<const double*>(L.d_x), z, n);
+  return cudaGetLastError();
+}
+
+cudaError_t mg_issue(MG& mg, const double* r, double* z, cudaStream_t stream, int trans) {
+  const int t = trans ? 1 : 0;
+  cudaError_t e = mg_enter(mg, r, stream);
+  if (e == cudaSuccess)
+    e = mg.precision == kPrecF32 ? issue_vcycle<float>(mg, 0, stream, t) : issue_vcycle<double>(mg, 0, stream, t);
+  return e == cudaSuccess ? mg_leave(mg, z, stream) : e;
+}
+
 cudaError_t mg_apply(MG& mg, const double* r, double* z, cudaStream_t stream, int trans) {
-  MGLevel& L0 = mg.lv[0];
-  const long long n = (long long)L0.hp.n_xi * L0.hp.n_t * L0.hp.n_x;
   const bool f32 = mg.precision == kPrecF32;
   const int t = trans ? 1 : 0;
   cudaError_t e;
@@ -1779,17 +1955,9 @@ cudaError_t mg_apply(MG& mg, const double* r, double* z, cudaStream_t stream, in
     if (e != cudaSuccess) return e;
     if ((e = cudaGraphInstantiate(&mg.exec_t[t], mg.graph_t[t], 0)) != cudaSuccess) return e;
   }
-  if (f32)
-    mg_convert<double, float><<<grid_for(n, 256), 256, 0, stream>>>(r, static_cast<float*>(L0.d_b), n);
-  else
-    mg_convert<double, double><<<grid_for(n, 256), 256, 0, stream>>>(r, static_cast<double*>(L0.d_b), n);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = mg_enter(mg, r, stream)) != cudaSuccess) return e;
   if ((e = cudaGraphLaunch(mg.exec_t[t], stream)) != cudaSuccess) return e;
-  if (f32)
-    mg_convert<float, double><<<grid_for(n, 256), 256, 0, stream>>>(static_cast<const float*>(L0.d_x), z, n);
-  else
-    mg_convert<double, double><<<grid_for(n, 256), 256, 0, stream>>>(static_cast<const double*>(L0.d_x), z, n);
-  return cudaGetLastError();
+  return mg_leave(mg, z, stream);
 }
 
 }  // namespace sg

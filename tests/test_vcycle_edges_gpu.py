@@ -23,6 +23,7 @@ def _spec(cells, k, r, M, P, hi, coef=None):
 CASES = {
     "2d-q2-20x12-dg1": _spec((20, 12), 2, 1, 2, 2, (1.0, 0.7)),           # 6 rows, 33-node lines over two warps
     "2d-q2-36x4-dg0": _spec((36, 4), 2, 0, 2, 2, (1.0, 1.0)),             # a row longer than a warp
+    "2d-q2-512x8-dg0": _spec((512, 8), 2, 0, 1, 0, (1.0, 1.0)),           # transfer rows beyond 48 KB of shared memory
     "2d-q1-12x20-dg2": _spec((12, 20), 1, 2, 3, 1, (0.4, 1.0)),
     "2d-q3-8x6-dg3-classes": _spec((8, 6), 3, 3, 4, 2, (0.5, 0.5), I.paper_coefficient()),
     "3d-q2-6x4x8": _spec((6, 4, 8), 2, 1, 2, 1, (1.0, 0.5, 0.8)),
