@@ -156,8 +156,8 @@ typedef struct {
   int max_slab_iterations; /* largest per-slab iteration count               */
   double max_rel_residual; /* largest final relative residual of a slab      */
   double solve_ms;         /* wall time of the call                          */
-  int tile;                /* samples per tile of the apply (autotuned)      */
-  int chunk;               /* cells per chunk of the apply (autotuned)       */
+  int tile;                /* samples per tile of the apply                  */
+  int chunk;               /* cells a warp of the apply takes               */
 } sg_mc_stats;
 
 /* Statistics of one sg_adjoint_gradient call (host struct out). */
@@ -496,8 +496,8 @@ sg_status sg_stat_errors(sg_ctx* ctx, const double* mean, const double* var, dou
  * preconditioner.  Samples are split into groups solved one after another
  * only when the device memory cannot hold them at once.
  *   xi        HOST n_samples x M standard-normal samples
- *   batch     samples per tile of the apply launch, 1..512 (reduced to fit
- *             shared memory)
+ *   batch     samples per tile of the apply launch, 1..512 (an apply
+ *             launch covers whole tiles)
  *   mg_precision  SG_PREC_FP64, SG_PREC_FP32 or SG_PREC_BF16 V-cycle
  *   mean_T, var_T  DEVICE n_x doubles out: nodal sample mean and unbiased
  *             sample variance of u(x, T)

@@ -11,7 +11,6 @@ namespace sg {
 cudaError_t bounds_fetch_apply_f64(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_apply_dw(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_apply_f32(BoundsRecord* out, bool clear);
-cudaError_t bounds_fetch_mc_apply(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_diag(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_mg(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_factor(BoundsRecord* out, bool clear);
@@ -50,7 +49,7 @@ sg_status sg_debug_bounds(int* enabled, unsigned int* count, int* site, long lon
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return fail(SG_ERR_CUDA, "sg_debug_bounds: synchronize failed");
   cudaError_t (*const fetch[])(sg::BoundsRecord*, bool) = {
-      sg::bounds_fetch_apply_f64, sg::bounds_fetch_apply_dw, sg::bounds_fetch_apply_f32, sg::bounds_fetch_mc_apply,
+      sg::bounds_fetch_apply_f64, sg::bounds_fetch_apply_dw, sg::bounds_fetch_apply_f32,
       sg::bounds_fetch_mg,        sg::bounds_fetch_factor,   sg::bounds_fetch_debug, sg::bounds_fetch_vanka_tc,
       sg::bounds_fetch_diag};
   for (auto f : fetch) {

@@ -30,6 +30,7 @@ namespace sg {
 namespace {
 
 constexpr int kDiagRows = 4;   // rows (warps) per block
+static_assert(kDiagCells == 32, "a lane per cell");
 
 template <typename T>
 struct DiagArgs {
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
     const T* src = p.x + (v0 + i) * p.n_x;
 #pragma unroll
     for (int a = 0; a < NQD; ++a)
-      v[i][a] = inner(a) && SG_IN((v0 + i) * p.n_x + offset(a), n_vec, 601) ? __ldg(src + offset(a)) : T(0);
+      v[i][a] = inner(a) && SG_IN((v0 + i) * p.n_x + offset(a), n_vec, 701) ? __ldg(src + offset(a)) : T(0);
   }
   // the row's coefficient at the cell's points
   T c[NQD];
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
     }
 #pragma unroll
     for (int a = 0; a < NQD; ++a)
-      if (inner(a) && !(a % N == K && give) && SG_IN((v0 + i) * p.n_x + offset(a), n_vec, 602))
+      if (inner(a) && !(a % N == K && give) && SG_IN((v0 + i) * p.n_x + offset(a), n_vec, 702))
         A::add_out(dst + offset(a), A::mul(p.tb[i], r[a]));
   }
 }

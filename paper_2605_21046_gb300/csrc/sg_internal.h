@@ -155,45 +155,13 @@ cudaError_t launch_apply(const HostProblem& hp, const LaunchShape& ls, const App
 // Kernel attribute set-up (max dynamic shared memory).
 cudaError_t prepare_apply_kernel(int precision, int dim, int k, int n_t, size_t smem);
 
-// ---------------------------------------------------------------- Monte-Carlo apply
-// One pathwise problem family of a Monte-Carlo apply launch: S samples of the
-// deterministic slab operator A_t (x) M + B_t (x) K[a(., xi_s)] on one mesh.
-constexpr int kMcMaxProb = 4;
-struct McProblem {
-  const void* x;             // S x N_t x n_x input (IO type of the arithmetic)
-  void* y;                   // output
-  const void* b;             // right-hand side of the residual / accumulate modes
-  const double* ctab;        // [cell][term][NQD]: w_q |J| a_t(x_q) / h_0^2
-  const double* wgt;         // [S][n_terms]: Psi_t(xi_s)
-  const double* amq;         // [NQD][N_t][N_t]: w_q |J| T[i][j] / (tau Bhat_ii)
-  long long n_x;
-  long long unit0;           // first work unit (cell x sample tile) of this problem
-  int n_cells, S, ts, tiles;
-  int nn[3], cells[3];
-  int aniso;
-  double ratio[3];
-};
 // Bytes of y rows one Monte-Carlo apply launch covers (whole sample tiles):
 // preset and then reduced into while they stay in L2.
 constexpr double kMcWaveBytes = 64.0 * 1024 * 1024;
 
-struct McParams {
-  McProblem pr[kMcMaxProb];
-  int n_prob, n_terms, chunk, mode, mass_only;
-  long long units;
-  long long u_lo = 0, u_hi = -1;   // units of this launch (whole sample tiles); u_hi < 0: all of them
-  int bd_zero = 0;                  // residual whose x equals b on the boundary: its Dirichlet rows are 0
-  double tb[kMaxNT];
-};
-// Shared memory of the Monte-Carlo apply for a chunk of cells and a sample tile.
-size_t mc_smem_bytes(int dim, int k, int n_t, int ts, int n_terms, int chunk, int value_bytes);
 // w_q |J| T[i][j] / (tau Bhat_ii) for one mesh (T = A_hat, its transpose, or C_t).
 void mc_amq(const HostProblem& hp, const std::vector<double>& T, std::vector<double>& amq);
-// Launches the init kernels of every problem and one Monte-Carlo apply.
-cudaError_t launch_mc_apply(int precision, int dim, int k, int n_t, const McParams& p, int grid, int threads,
-                            size_t smem, cudaStream_t s);
-// Kernel attribute set-up for the Monte-Carlo apply of one shape.
-cudaError_t prepare_mc_kernel(int precision, int dim, int k, int n_t);
+constexpr int kMcMaxProb = 4;   // meshes of one Monte-Carlo system
 
 // Precision of the apply kernels used inside the multigrid preconditioner.
 constexpr int kPrecF32 = SG_PREC_FP32;
@@ -213,6 +181,7 @@ struct DiagParams {
   int cells[3], nn[3];
   double ratio[3], tb[kMaxNT];
 };
+constexpr int kDiagCells = 32;   // cells of a warp
 cudaError_t launch_diag_apply(int precision, int dim, int k, int n_t, const DiagParams& p, cudaStream_t s);
 // The coefficient of the terms `used` as [term][NQD][cell] in the given
 // precision (allocates *out; synchronous).

@@ -4,9 +4,8 @@
 // mc-variance-estimator-unbiased, and Algorithm 1).
 //
 // All samples of all meshes of a call form ONE block-diagonal system per
-// slab: the Monte-Carlo apply (sg_mc_apply.cu) evaluates every pathwise
-// operator A(xi_s) = A_t (x) M + B_t (x) K[a(., xi_s)] of every mesh in one
-// launch over a queue of (mesh, sample tile, cell) units, the right-hand side
+// slab: the row-diagonal apply (sg_diag.cu) evaluates every pathwise operator
+// A(xi_s) = A_t (x) M + B_t (x) K[a(., xi_s)], the right-hand side
 // of sample s is the manufactured forcing f(x, t, xi_s) (its load vector is
 // combined on the device from spatial tables per distinct spatial factor of
 // the exact solution), and one FGMRES iterates on the whole system.  The
@@ -27,6 +26,7 @@
 #include <vector>
 
 #include "sg_internal.h"
+#include "sg_vec.cuh"
 
 namespace sg {
 
@@ -225,7 +225,9 @@ struct McMesh {
   HostProblem hp;
   ExactData* E = nullptr;
   MG* mg = nullptr;
-  double *d_wgt = nullptr, *d_amqA = nullptr, *d_amqC = nullptr;
+  double* d_wgt = nullptr;
+  void* d_coef = nullptr;              // coefficient of the row-diagonal apply
+  std::vector<double> amqA, amqC;      // its time-mass tables: apply and transfer
   long long off = 0, n = 0;
   double n_done = 0.0;
 };
@@ -249,6 +251,22 @@ void free_group(McMesh& m) {
 }
 
 }  // namespace
+
+void mc_amq(const HostProblem& hp, const std::vector<double>& Tm, std::vector<double>& amq) {
+  const int nq = hp.k + 1, nqd = hp.dim == 2 ? nq * nq : nq * nq * nq, nt = hp.n_t;
+  double detJ = 1.0;
+  for (int d = 0; d < hp.dim; ++d) detJ *= hp.h[d];
+  amq.assign((size_t)nqd * nt * nt, 0.0);
+  for (int qd = 0; qd < nqd; ++qd) {
+    const int qi[3] = {qd % nq, (qd / nq) % nq, qd / (nq * nq)};
+    double w = detJ;
+    for (int d = 0; d < hp.dim; ++d) w *= hp.wq[qi[d]];
+    for (int i = 0; i < nt; ++i) {
+      const double tb = hp.tau * hp.B_hat[i * nt + i];
+      for (int j = 0; j < nt; ++j) amq[((size_t)qd * nt + i) * nt + j] = w * Tm[(size_t)i * nt + j] / tb;
+    }
+  }
+}
 
 sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector<int>& n_samples,
                           const std::vector<const double*>& xis, int tile, int mg_precision, double rtol, int max_it,
@@ -295,7 +313,7 @@ sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector
       }
     }
     m.ng = (int)gfreq.size();
-    std::vector<double> Pg, Kg, amqA, amqC;
+    std::vector<double> Pg, Kg;
     spatial_tables(m.parent->hp, gfreq, Pg, Kg);
     if (e == cudaSuccess) e = cudaMalloc(&m.d_Pg, Pg.size() * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&m.d_Kg, Kg.size() * sizeof(double));
@@ -307,38 +325,17 @@ sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector
     std::vector<double> Ct((size_t)nt * nt);
     for (int i = 0; i < nt; ++i)
       for (int j = 0; j < nt; ++j) Ct[(size_t)i * nt + j] = lagrange(nodes, i, 0.0) * lagrange(nodes, j, 1.0);
-    mc_amq(h, h.A_hat, amqA);
-    mc_amq(h, Ct, amqC);
-    if (e == cudaSuccess) e = cudaMalloc(&m.d_amqA, amqA.size() * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&m.d_amqC, amqC.size() * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemcpy(m.d_amqA, amqA.data(), amqA.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(m.d_amqC, amqC.data(), amqC.size() * sizeof(double), cudaMemcpyHostToDevice);
+    mc_amq(h, h.A_hat, m.amqA);
+    mc_amq(h, Ct, m.amqC);
+    std::vector<int> terms(nterm);
+    for (int t = 0; t < nterm; ++t) terms[t] = t;
+    if (e == cudaSuccess) e = diag_coefficients(SG_PREC_FP64, h, m.parent->d_ctab, terms, &m.d_coef, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(mean_T[p], 0, h.n_x * sizeof(double), stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(var_T[p], 0, h.n_x * sizeof(double), stream);
   }
-  // apply tile shapes: (samples per tile, cells per chunk) candidates within the
-  // shared-memory budget; the fastest on the first group's system is kept
-  struct Shape2 {
-    int ts, chunk;
-    size_t smem;
-  };
-  std::vector<Shape2> cand;
-  for (int t = 8; t <= std::max(8, tile); t *= 2) {
-    const int tt = std::min(t, std::max(1, tile));
-    int best_c = 0;
-    for (int c = 1; c <= 8; ++c)
-      if (mc_smem_bytes(h0.dim, h0.k, nt, tt, nterm, c, 8) <= 100 * 1024) best_c = c;
-    if (best_c == 0) break;
-    cand.push_back({tt, best_c, mc_smem_bytes(h0.dim, h0.k, nt, tt, nterm, best_c, 8)});
-    if (best_c > 2) cand.push_back({tt, best_c / 2, mc_smem_bytes(h0.dim, h0.k, nt, tt, nterm, best_c / 2, 8)});
-    if (tt == tile) break;
-  }
-  if (cand.empty()) cand.push_back({1, 1, mc_smem_bytes(h0.dim, h0.k, nt, 1, nterm, 1, 8)});
-  int ts = cand.back().ts, chunk = cand.back().chunk;
-  size_t smem = cand.back().smem;
-  bool tuned = cand.size() == 1;
+  stats.tile = std::min(tile, *std::max_element(n_samples.begin(), n_samples.end()));
+  stats.chunk = kDiagCells;
   stats.max_rel_residual = 0.0;
-  if (e == cudaSuccess) e = prepare_mc_kernel(SG_PREC_FP64, h0.dim, h0.k, nt);
   // sample groups: all samples in one system unless the device memory says otherwise
   const int m_restart = 10;
   double vec_bytes = 0.0;
@@ -431,69 +428,44 @@ sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&d_krylov), krylov_bytes(N, m_restart));
     if (e == cudaSuccess) e = cudaMemsetAsync(U, 0, N * sizeof(double), stream);
     if (e != cudaSuccess) break;
-    McParams base;
-    long long units = 0;
-    int grid = 1;
-    auto build_base = [&]() {
-      std::memset(&base, 0, sizeof(base));
-      base.u_hi = -1;
-      units = 0;
-      for (int p = 0; p < P; ++p) {
-        McMesh& m = ms[p];
-        if (m.S == 0) continue;
-        McProblem& pr = base.pr[base.n_prob++];
-        const HostProblem& ph = m.parent->hp;
-        pr.ctab = m.parent->d_ctab;
-        pr.wgt = m.d_wgt;
-        pr.n_x = ph.n_x;
-        pr.unit0 = units;
-        pr.n_cells = (int)ph.n_cells;
-        pr.S = m.S;
-        pr.ts = std::min(ts, m.S);
-        pr.tiles = (m.S + pr.ts - 1) / pr.ts;
-        for (int d = 0; d < 3; ++d) {
-          pr.nn[d] = ph.nn[d];
-          pr.cells[d] = ph.cells[d];
-          pr.ratio[d] = d < ph.dim ? (ph.h[0] * ph.h[0]) / (ph.h[d] * ph.h[d]) : 0.0;
-        }
-        pr.aniso = 0;
-        for (int d = 1; d < ph.dim; ++d) pr.aniso |= ph.h[d] != ph.h[0];
-        units += (long long)pr.tiles * pr.n_cells;
-      }
-      base.n_terms = nterm;
-      base.chunk = chunk;
-      base.units = units;
-      for (int i = 0; i < nt; ++i) base.tb[i] = h0.tau * h0.B_hat[i * nt + i];
-      grid = (int)std::max<long long>(1, std::min<long long>(units / chunk, sg::sm_count() * 2));
-    };
-    build_base();
+    // Row-diagonal apply of every mesh, in waves of whole sample tiles whose
+    // rows of y (preset, then reduced into by the apply) stay resident in L2
+    // between the two
     auto mc_launch = [&](const double* x, double* y, const double* b, int mode, bool transfer,
                          cudaStream_t st) -> cudaError_t {
-      McParams q = base;
-      q.mode = mode;
-      q.mass_only = transfer ? 1 : 0;
-      int j = 0;
-      for (int p = 0; p < P; ++p) {
+      cudaError_t err = cudaSuccess;
+      for (int p = 0; p < P && err == cudaSuccess; ++p) {
         McMesh& m = ms[p];
         if (m.S == 0) continue;
-        q.pr[j].x = x + m.off;
-        q.pr[j].y = y + m.off;
-        q.pr[j].b = b ? b + m.off : nullptr;
-        q.pr[j].amq = transfer ? m.d_amqC : m.d_amqA;
-        ++j;
-      }
-      // waves of whole sample tiles whose rows of y (preset, then reduced into
-      // by the apply) stay resident in L2 between the two
-      cudaError_t err = cudaSuccess;
-      for (int pi = 0; pi < base.n_prob && err == cudaSuccess; ++pi) {
-        const McProblem& P = base.pr[pi];
-        const double tile_bytes = (double)P.ts * nt * P.n_x * sizeof(double);
-        const int tpw = std::max(1, (int)(kMcWaveBytes / tile_bytes));
-        for (int t0 = 0; t0 < P.tiles && err == cudaSuccess; t0 += tpw) {
-          q.u_lo = P.unit0 + (long long)t0 * P.n_cells;
-          q.u_hi = P.unit0 + (long long)std::min(P.tiles, t0 + tpw) * P.n_cells;
-          const int g = (int)std::max<long long>(1, std::min<long long>((q.u_hi - q.u_lo) / chunk, grid));
-          err = launch_mc_apply(SG_PREC_FP64, h0.dim, h0.k, nt, q, g, 256, smem, st);
+        const HostProblem& ph = m.parent->hp;
+        DiagParams q;
+        std::memset(&q, 0, sizeof(q));
+        q.ctab = m.d_coef;
+        q.amq = (transfer ? m.amqC : m.amqA).data();
+        q.sign = 1.0;
+        q.n_x = ph.n_x;
+        q.n_cells = (int)ph.n_cells;
+        q.n_terms = nterm;
+        q.mass_only = transfer ? 1 : 0;
+        for (int d = 0; d < 3; ++d) {
+          q.nn[d] = ph.nn[d];
+          q.cells[d] = ph.cells[d];
+          q.ratio[d] = d < ph.dim ? (ph.h[0] * ph.h[0]) / (ph.h[d] * ph.h[d]) : 1.0;
+        }
+        for (int i = 0; i < nt; ++i) q.tb[i] = h0.tau * h0.B_hat[i * nt + i];
+        const long long row = (long long)nt * ph.n_x;
+        const int ts = std::min(tile, m.S);
+        const int wave = std::max(1, (int)(kMcWaveBytes / ((double)ts * row * sizeof(double)))) * ts;
+        for (int s0 = 0; s0 < m.S && err == cudaSuccess; s0 += wave) {
+          const int rows = std::min(wave, m.S - s0);
+          const long long off = m.off + s0 * row;
+          launch_vec_start<double>(b ? b + off : nullptr, x + off, y + off, mode == kApplyAccumulate ? 3 : 2, rows * nt,
+                                   ph.n_x, ph.nn, ph.dim, st);
+          q.x = x + off;
+          q.y = y + off;
+          q.wgt = m.d_wgt + (size_t)s0 * nterm;
+          q.rows = rows;
+          err = launch_diag_apply(SG_PREC_FP64, ph.dim, ph.k, nt, q, st);
         }
       }
       return err;
@@ -501,42 +473,6 @@ sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector
     auto apply = [&](const double* in, double* out, cudaStream_t st) {
       return mc_launch(in, out, nullptr, kApplyPlain, false, st);
     };
-    if (!tuned) {
-      // time one apply per candidate shape (after one untimed launch) on this system
-      cudaEvent_t ea = nullptr, eb = nullptr;
-      e = cudaEventCreate(&ea);
-      if (e == cudaSuccess) e = cudaEventCreate(&eb);
-      float best_ms = 1e30f;
-      Shape2 best = cand.back();
-      for (const Shape2& c : cand) {
-        if (e != cudaSuccess) break;
-        ts = c.ts;
-        chunk = c.chunk;
-        smem = c.smem;
-        build_base();
-        e = apply(U, RHS, stream);
-        if (e == cudaSuccess) e = cudaEventRecord(ea, stream);
-        if (e == cudaSuccess) e = apply(U, RHS, stream);
-        if (e == cudaSuccess) e = cudaEventRecord(eb, stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(eb);
-        float ms = 0.0f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ea, eb);
-        if (e == cudaSuccess && ms < best_ms) {
-          best_ms = ms;
-          best = c;
-        }
-      }
-      if (ea) cudaEventDestroy(ea);
-      if (eb) cudaEventDestroy(eb);
-      ts = best.ts;
-      chunk = best.chunk;
-      smem = best.smem;
-      build_base();
-      tuned = true;
-      stats.tile = ts;
-      stats.chunk = chunk;
-      if (e != cudaSuccess) break;
-    }
     auto prec = [&](const double* in, double* out, cudaStream_t st) -> cudaError_t {
       for (int p = 0; p < P; ++p) {
         McMesh& m = ms[p];
@@ -584,8 +520,7 @@ sg_status mc_solve_meshes(const std::vector<sg_ctx*>& parents, const std::vector
     free_group(m);
     cudaFree(m.d_Pg);
     cudaFree(m.d_Kg);
-    cudaFree(m.d_amqA);
-    cudaFree(m.d_amqC);
+    cudaFree(m.d_coef);
   }
   cudaFree(U);
   cudaFree(RHS);
