@@ -457,6 +457,7 @@ __global__ void __launch_bounds__(256, 2) mg_vanka(const VankaParams<T> p) {
 // on the boundary for the residual that follows.
 constexpr int kAxisMax = 16;  // entries of one output of a 1D transfer list, at most (4k + 1 for k <= 3)
 constexpr int kTransferThreads = 256;
+constexpr int kTransferBatch = 4;   // elements of a thread whose loads are in flight together
 
 template <typename T>
 struct TransferParams {
@@ -491,16 +492,35 @@ __device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz
       pl[k] = src + (long long)__ldg(p.idx[2] + k * p.no[2] + jz) * plane + off;
       if (wk != T(0)) m = k + 1;
     }
-    for (int i = threadIdx.x; i < n; i += kTransferThreads) {
-      T s = T(0);
+    for (int i0 = threadIdx.x; i0 < n; i0 += kTransferBatch * kTransferThreads) {
+      T s[kTransferBatch];
 #pragma unroll
-      for (int k = 0; k < W; ++k)
-        if (k < m && SG_IN(pl[k] - p.in + i, p.lim_in, 501)) s = fma(wz[k], __ldg(pl[k] + i), s);
-      S0[i] = s;
+      for (int g = 0; g < kTransferBatch; ++g) s[g] = T(0);
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        if (k >= m) break;
+#pragma unroll
+        for (int g = 0; g < kTransferBatch; ++g) {
+          const int i = i0 + g * kTransferThreads;
+          if (i < n && SG_IN(pl[k] - p.in + i, p.lim_in, 501)) s[g] = fma(wz[k], __ldg(pl[k] + i), s[g]);
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < kTransferBatch; ++g)
+        if (i0 + g * kTransferThreads < n) S0[i0 + g * kTransferThreads] = s[g];
     }
   } else {
-    for (int i = threadIdx.x; i < n; i += kTransferThreads)
-      if (SG_IN(v_in + off + i, p.lim_in, 501)) S0[i] = __ldg(src + off + i);
+    for (int i0 = threadIdx.x; i0 < n; i0 += kTransferBatch * kTransferThreads) {
+      T s[kTransferBatch];
+#pragma unroll
+      for (int g = 0; g < kTransferBatch; ++g) {
+        const int i = i0 + g * kTransferThreads;
+        s[g] = i < n && SG_IN(v_in + off + i, p.lim_in, 501) ? __ldg(src + off + i) : T(0);
+      }
+#pragma unroll
+      for (int g = 0; g < kTransferBatch; ++g)
+        if (i0 + g * kTransferThreads < n) S0[i0 + g * kTransferThreads] = s[g];
+    }
   }
 }
 
@@ -567,6 +587,7 @@ __global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferPar
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][coarse x]
   T* S1 = S0 + (size_t)p.max_rows * p.ni[0];                    // [tile][coarse x]
+  T* S2 = S1 + (size_t)p.tile * p.ni[0];                        // [tile][fine x]
   const int jz = blockIdx.y, j0 = blockIdx.z * p.tile, nj = min(p.tile, p.no[1] - j0);
   const int lo = __ldg(p.range + 2 * blockIdx.z), cnt = __ldg(p.range + 2 * blockIdx.z + 1);
   transfer_load<T, W>(p, jz, lo, cnt, S0);
@@ -575,16 +596,32 @@ __global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferPar
   transfer_pass<T, W, 1>(S0, ncx, ncx, p.cb_in, nj, p.idx[1], p.w[1], p.no[1], j0, lo,
                          [&](int r, int c, T v) { S1[r * ncx + c] = v; });
   __syncthreads();
+  transfer_pass<T, W, 0>(S1, ncx, nfx, p.cb_out, nj, p.idx[0], p.w[0], nfx, 0, 0,
+                         [&](int r, int c, T v) { S2[r * nfx + c] = v; });
+  __syncthreads();
+  // the tile's rows are contiguous: x += S2, r = b inside, with the loads of a batch in flight together
   const long long o0 = (long long)blockIdx.x * p.n_out + ((long long)jz * p.no[1] + j0) * nfx;
   const bool edge_z = p.z && (jz == 0 || jz == p.no[2] - 1);
-  transfer_pass<T, W, 0>(S1, ncx, nfx, p.cb_out, nj, p.idx[0], p.w[0], nfx, 0, 0, [&](int r, int c, T v) {
-    const long long o = o0 + (long long)r * nfx + c;
-    if (!SG_IN(o, p.lim_out, 503)) return;
-    const int jy = j0 + r;
-    const bool bd = edge_z || jy == 0 || jy == p.no[1] - 1 || c == 0 || c == nfx - 1;
-    p.out[o] += v;
-    p.r[o] = bd ? T(0) : p.b[o];
-  });
+  const int n = nj * nfx;
+  for (int i0 = threadIdx.x; i0 < n; i0 += kTransferBatch * kTransferThreads) {
+    T xv[kTransferBatch], bv[kTransferBatch];
+#pragma unroll
+    for (int g = 0; g < kTransferBatch; ++g) {
+      const int i = i0 + g * kTransferThreads;
+      const bool in = i < n && SG_IN(o0 + i, p.lim_out, 503);
+      xv[g] = in ? p.out[o0 + i] : T(0);
+      bv[g] = in ? __ldg(p.b + o0 + i) : T(0);
+    }
+#pragma unroll
+    for (int g = 0; g < kTransferBatch; ++g) {
+      const int i = i0 + g * kTransferThreads;
+      if (i >= n || !SG_IN(o0 + i, p.lim_out, 503)) continue;
+      const int r = i / nfx, c = i - r * nfx, jy = j0 + r;
+      const bool bd = edge_z || jy == 0 || jy == p.no[1] - 1 || c == 0 || c == nfx - 1;
+      p.out[o0 + i] = xv[g] + S2[i];
+      p.r[o0 + i] = bd ? T(0) : bv[g];
+    }
+  }
 }
 
 // Coarsest level: x[inner] = inv(C_class) b[inner] for every chaos mode
@@ -1170,9 +1207,10 @@ void transfer_params(const MGLevel& I, const MGLevel& O, const MGLevel::Transfer
 }
 
 // Bytes of shared memory of a transfer block: the input rows, and the rows
-// between its two passes (restriction: the input rows; interpolation: the tile).
+// between its passes (restriction: the input rows; interpolation: the tile,
+// with coarse and then fine rows).
 size_t transfer_smem(bool up, int max_rows, int tile, int nfx, int ncx, size_t vb) {
-  return vb * (up ? (size_t)max_rows * ncx + (size_t)tile * ncx : (size_t)max_rows * (nfx + ncx));
+  return vb * (up ? (size_t)max_rows * ncx + (size_t)tile * (ncx + nfx) : (size_t)max_rows * (nfx + ncx));
 }
 
 #define SG_TRANSFER_WIDTHS(CALL) \
