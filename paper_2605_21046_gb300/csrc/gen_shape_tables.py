@@ -4,6 +4,10 @@ and ones out of the sum-factorisation passes.
 
   S[q][n]  = l_n(g_q): Gauss-Lobatto Lagrange basis l_n at the (k+1) Gauss points g_q
   D[q][p]  = L_p'(g_q): derivative of the Lagrange basis L_p on the Gauss points
+  L[i]     = the constants of the 1D passes of Q2 and Q3 (Line in sg_apply_kernel.cuh), in
+             the order of its enumerators, and W, the square of the unit its derivatives
+             are taken in; each rounded once (derived from S and D in double they cost Q3
+             half as much error again)
   Sh/Sl, Dh/Dl: the same values as float pairs hi + lo (hi = value rounded to
   float, lo = the remainder rounded to float), for double-word arithmetic
 
@@ -83,6 +87,22 @@ def table(name, n, vals, typ, fmt):
             "    return t[a][b];", "  }"]
 
 
+def line_constants(k, S, D):
+    """(constants, squared derivative unit) of the 1D passes."""
+    if k == 1:
+        return [mp.mpf(0)], mp.mpf(1)
+    if k == 2:
+        return [mp.mpf(3) / 10, mp.mpf(4) / 10, (S[2][2] - S[2][0]) / 2, mp.mpf(12) / 10], D[1][2] ** 2
+    unit = (D[3][3] - D[3][0]) / 2
+    even = lambda T, q, n: (T[q][n] + T[q][3 - n]) / 2  # noqa: E731
+    odd = lambda T, q, n: (T[q][n] - T[q][3 - n]) / 2  # noqa: E731
+    co, ci, co1, ci0 = odd(S, 3, 3), odd(S, 2, 2), odd(S, 3, 2), odd(S, 2, 3)
+    qo, qi = even(D, 3, 3) / unit, even(D, 2, 3) / unit
+    ai, bo, bi = odd(D, 2, 3) / unit, odd(D, 3, 2) / unit, odd(D, 2, 2) / unit
+    return [even(S, 3, 3), even(S, 3, 2), even(S, 2, 3), even(S, 2, 2), co, ci, co1 / co, ci0 / ci, ci0 / co, co1 / ci,
+            ai, bo, bi, qo, qi, 2 * qo, 2 * qi, 2 * ai, 2 * bo, 2 * bi], unit ** 2
+
+
 def main():
     out = ["// Generated by gen_shape_tables.py - do not edit.",
            "// Reference Q_k tables on [0,1] at the (k+1)-point Gauss rule.",
@@ -115,6 +135,11 @@ def main():
         out += table("Sl", n, Sl, "float", flit)
         out += table("Dh", n, Dh, "float", flit)
         out += table("Dl", n, Dl, "float", flit)
+        L, W = line_constants(k, S, D)
+        out += [f"  static constexpr double W = {lit(W)};",
+                "  __host__ __device__ static constexpr double L(int i) {",
+                f"    constexpr double t[{len(L)}] = {{{', '.join(lit(v) for v in L)}}};",
+                "    return t[i];", "  }"]
         out.append("};")
         out.append("")
     out.append("}  // namespace sg")

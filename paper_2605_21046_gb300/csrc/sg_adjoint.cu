@@ -51,6 +51,7 @@ struct BilinParams {
   int n_xi, n_terms, n_tab, nnz, chunk, cell_tab;
   double tb[kMaxNT];
   double ratio[3];
+  double lk[kLineConsts];
   double* out_sum;          // [n_tab] += sum over cells
   double* out_cell;         // [n_cells] += the per-cell value of table cell_tab (or null)
 };
@@ -64,12 +65,14 @@ size_t bilin_smem(int dim, int k, int n_t, int n_xi, int nnz, int n_tab, int chu
 }
 
 template <int DIM, int K, int NT>
-__global__ void __launch_bounds__(256) k_bilinear(const BilinParams p) {
+__global__ void __launch_bounds__(256) k_bilinear(const __grid_constant__ BilinParams p) {
   using Sh = Shape<DIM, K>;
   constexpr int NQD = Sh::NQD, NKD = Sh::NKD, NC = Sh::NC, N = Sh::N;
   constexpr int SLOT = NC * NQD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double s_lk[kLineConsts];
   const int tid = threadIdx.x, nthr = blockDim.x;
+  if (tid < kLineConsts) s_lk[tid] = p.lk[tid];   // visible after the first barrier
   const int n_xi = p.n_xi, V = n_xi * NT, C = p.chunk;
   double* Ql = reinterpret_cast<double*>(smem_raw);         // [C][V][NC][NQD]
   double* Qu = Ql + (size_t)C * V * SLOT;
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(256) k_bilinear(const BilinParams p) {
       double u[NKD];
 #pragma unroll
       for (int a = 0; a < NKD; ++a) u[a] = q[a];
-      forward_cell<F64, DIM, K>(u, [&](int o, double v) { q[o] = v; });
+      forward_cell<F64, DIM, K>(Line<F64, K>(s_lk), u, [&](int o, double v) { q[o] = v; });
     }
     __syncthreads();
     for (int it = tid; it < nc * NQD * n_xi; it += nthr) {
@@ -345,6 +348,7 @@ sg_status adjoint_gradient(sg_ctx* ctx, double rtol, int max_it, int K, int cell
   // backward sweep by segments
   BilinParams bp;
   std::memset(&bp, 0, sizeof(bp));
+  fill_line_consts(hp.k, bp.lk);
   int bchunk = 0;
   {
     int dev = 0, optin = 0;
@@ -353,7 +357,7 @@ sg_status adjoint_gradient(sg_ctx* ctx, double rtol, int max_it, int K, int cell
     for (int c = 1; c <= 16; ++c)
       if (bilin_smem(hp.dim, hp.k, nt, hp.n_xi, (int)hp.g.col.size(), n_tab, c) <= (size_t)optin - 1024) bchunk = c;
     if (bchunk == 0) { msg = "gradient kernel does not fit in shared memory"; status = SG_ERR_UNSUPPORTED; }
-    else e = cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    else e = cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
   }
   bp.dtab = d_dtab;
   bp.tab_term = d_tt;

@@ -50,6 +50,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include "sg_apply_kernel.cuh"
 #include "sg_internal.h"
 #include "sg_shape_tables.h"
 #include "sg_vec.cuh"
@@ -121,7 +122,8 @@ static void* select_kernel(int precision, int dim, int k, int n_t) {
 
 // The dynamic shared-memory limit is a property of the kernel function, shared
 // by every context and multigrid level that launches it: it is always set to
-// the device's opt-in maximum, so a later set-up can never shrink the limit
+// the device's opt-in maximum (less the kernel's static shared memory, which
+// the 1 KB that plans leave covers), so a later set-up can never shrink the limit
 // below what an earlier one launches with.
 cudaError_t prepare_apply_kernel(int precision, int dim, int k, int n_t, size_t smem) {
   void* f = select_kernel(precision, dim, k, n_t);
@@ -129,7 +131,11 @@ cudaError_t prepare_apply_kernel(int precision, int dim, int k, int n_t, size_t 
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if ((size_t)optin < smem) return cudaErrorInvalidValue;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, f);
+  if (e != cudaSuccess) return e;
+  optin -= (int)fa.sharedSizeBytes;
+  if (optin < 0 || (size_t)optin < smem) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
 }
 
@@ -257,8 +263,10 @@ void fill_apply_params(const HostProblem& hp, const LaunchShape& ls, const void*
     const int n = coupling_pairs(hp, p.pair_term, p.pair_val);
     p.premul = n >= 0;
     p.n_pairs = n >= 0 ? n : 0;
+    for (int k = 0; k < p.n_pairs; ++k) p.pair_w[k] = grad_weight(hp.k) * p.pair_val[k];
   }
   p.stagger = ls.stagger;
+  fill_line_consts(hp.k, p.lk);
   const int nq = hp.k + 1;
   const int nqd = hp.dim == 2 ? nq * nq : nq * nq * nq;
   double detJ = 1.0;

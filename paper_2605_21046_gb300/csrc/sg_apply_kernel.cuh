@@ -4,6 +4,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "sg_arith.h"
 #include "sg_bounds.h"
 #include "sg_internal.h"
@@ -51,147 +53,217 @@ __device__ __forceinline__ typename A::T cdot(CF cf, XF xf) {
 // --------------------------------------------------------------- 1D lines
 // The passes of the sum factorisation along one line of N = K + 1 values.
 //
-// Derivatives are taken in units of deriv_scale<K>(): with the Gauss points'
+// Derivatives are taken in units of a unit of their own: with the Gauss points'
 // symmetry the collocation derivative needs few multiplies, and the remaining
 // common factor of every gradient is left out here and put back, squared, into
 // the coefficient (grad_weight<K>()), which multiplies each gradient once on
 // its way there and back.  FP64 instructions per line, dense tables against
 // this form: Q2 interpolation 6 / 6, derivative 8 / 4, their transposes 7 / 6
 // and 8 / 7, and 9 and 12 where one line needs value and derivative (15 and
-// 15); Q3 interpolation 16 / 14, derivative 16 / 12, transposes 16 / 14, both
+// 15); Q3 interpolation 16 / 14, derivative 16 / 12, transposes 16 / 14 and 16 / 18, both
 // at once 24 and 26 (32); Q1 derivative 4 / 2.  Double-word sums cost more than products (8 against
-// 4 instructions), so that arithmetic keeps the dense interpolation.  Bound by
-// the FP64 pipe (81 % active), the whole apply went from 186 to 165 us on 64^2
-// Q2 M=4 P=3, 3.36 to 3.02 ms on 32^3 Q2 M=3 P=3 and 1.79 to 1.62 ms on 128^2
-// Q3 dG(3); double-word 675 to 650 us on 128^2 Q2 M=4 P=4.  The error against
-// 64-bit references is the dense form's or less (Q2 4.5e-16 against 5.0e-16).
-template <int K>
-__host__ __device__ constexpr double deriv_scale() {
-  return K == 1 ? 1.0 : (K == 2 ? RefShape<2>::D(1, 2) : 0.5 * (RefShape<3>::D(3, 3) - RefShape<3>::D(3, 0)));
-}
-// deriv_scale squared: 1 (Q1 has one multiply to lose, and loses accuracy with
-// a rounded 3 a), 5/3, and the square of Q3's.
+// 4 instructions), so that arithmetic keeps the dense interpolation.  The
+// constants of the parts are rounded once from 40 digits (RefShape::L): formed
+// from the rounded tables they cost Q3 65 % more error.  Measured inside the
+// domain against an 80-bit reference, FP64 Q2 0.86e-15 (dense tables 1.02e-15),
+// Q3 3.5e-16 (3.7e-16), Q1 the same.
+// That weight is 1 for Q1 (which has one multiply to lose, and loses accuracy
+// with a rounded 3 a), 5/3 for Q2, and the square of Q3's unit.
 template <int K>
 __host__ __device__ constexpr double grad_weight() {
-  return K == 1 ? 1.0 : (K == 2 ? 5.0 / 3.0 : deriv_scale<3>() * deriv_scale<3>());
+  return RefShape<K>::W;
 }
-__host__ __device__ constexpr double grad_weight(int k) {
-  return k == 1 ? 1.0 : (k == 2 ? grad_weight<2>() : grad_weight<3>());
+inline double grad_weight(int k) {
+  return k == 1 ? RefShape<1>::W : (k == 2 ? RefShape<2>::W : RefShape<3>::W);
 }
 __host__ __device__ constexpr Cf cf_of(double c) {
   return {c, (float)c, (float)(c - (double)(float)c)};
+}
+
+// FP64 constants.  A GB300 SM takes 16.9 cycles per warp for a DFMA of three
+// registers but 20.0 for a DADD, a DMUL, or a DFMA with a literal or
+// constant-bank operand (measured; the kernels here sat at 82 % of the FP64
+// pipe at any occupancy).  So sums and products are written as fma(x, 1, y)
+// and fma(x, y, -0), which round the same, and every constant is read from a
+// shared-memory array, which forces it into a register.  64^2 Q2 165 -> 149 us,
+// 32^3 Q2 3.02 -> 2.73 ms, 128^2 Q3 dG(3) 1.62 -> 1.47 ms.
+enum { kOne, kNegZero, kTwo, kFour, kLineOwn };   // constants of every degree; then the degree's own
+// Q2: half the difference of the end functions at the outer Gauss point
+// (sqrt(3/5) / 2); their mean there is 0.3, the middle function 0.4.
+enum { kA2 = kLineOwn, kM2, kB2, kG2 };
+// Q3: even (E) and odd (C) parts of the end (0) and inner (1) basis functions
+// at the outer (o) and inner (i) Gauss points, ratios of the odd parts, and
+// the derivative's weights on (v3 - v0), (v2 - v1), (v0 + v3) - (v1 + v2).
+enum { kEo0 = kLineOwn, kEo1, kEi0, kEi1, kCo, kCi, kRo, kRi, kTo, kTi, kAi, kBo, kBi, kQo, kQi, kQo2, kQi2, kAi2, kBo2, kBi2 };
+
+template <int K>
+__host__ __device__ constexpr double line_const(int i) {
+  return i == kOne ? 1.0 : i == kNegZero ? -0.0 : i == kTwo ? 2.0 : i == kFour ? 4.0 : RefShape<K>::L(i - kLineOwn);
+}
+// The line constants of a degree as a kernel parameter (kLineConsts values).
+inline void fill_line_consts(int k, double* out) {
+  constexpr int n[4] = {0, kLineOwn, kG2 + 1, kBi2 + 1};
+  for (int i = 0; i < kLineConsts; ++i)
+    out[i] = i >= n[k] ? 0.0 : (k == 1 ? line_const<1>(i) : (k == 2 ? line_const<2>(i) : line_const<3>(i)));
 }
 
 template <class A, int K>
 struct Line {
   using T = typename A::T;
   static constexpr int N = K + 1;
+  static constexpr bool kF64 = std::is_same<A, F64>::value;
+  const double* k;   // the constants in shared memory
+  __device__ __forceinline__ explicit Line(const double* lk) : k(lk) {}
+
+  __device__ __forceinline__ double reg(int i) const { return k[i]; }
+  __device__ __forceinline__ T add(T a, T b) const {
+    if constexpr (kF64) return ::fma(a, reg(kOne), b);
+    else return A::add(a, b);
+  }
+  __device__ __forceinline__ T sub(T a, T b) const {
+    if constexpr (kF64) return ::fma(b, -reg(kOne), a);
+    else return A::add(a, A::neg(b));
+  }
+  __device__ __forceinline__ T mul(T a, T b) const {
+    if constexpr (kF64) return ::fma(a, b, reg(kNegZero));
+    else return A::mul(a, b);
+  }
+  // c x + y, -c x + y and c x for the constant I, as sums still to be finished (A::fin)
+  template <int I>
+  __device__ __forceinline__ T axpy(T x, T y) const {
+    if constexpr (kF64) {
+      return ::fma(reg(I), x, y);
+    } else {
+      A::cfma(cf_of(line_const<K>(I)), x, y);
+      return y;
+    }
+  }
+  template <int I>
+  __device__ __forceinline__ T axmy(T x, T y) const {
+    if constexpr (kF64) {
+      return ::fma(-reg(I), x, y);
+    } else {
+      A::cfma(cf_of(-line_const<K>(I)), x, y);
+      return y;
+    }
+  }
+  template <int I>
+  __device__ __forceinline__ T scale(T x) const {
+    if constexpr (kF64) return ::fma(reg(I), x, reg(kNegZero));
+    else return A::cmul(cf_of(line_const<K>(I)), x);
+  }
   template <class F>
   static __device__ __forceinline__ void dense(F c, const T* x, T* y) {
 #pragma unroll
     for (int a = 0; a < N; ++a)
       y[a] = cdot<A, N>([&](int j) { return c(a, j); }, [&](int j) { return x[j]; });
   }
-  // c x + y for a compile-time c, as a sum still to be finished (A::fin)
-  static __device__ __forceinline__ T axpy(Cf c, T x, T y) {
+  static __device__ __forceinline__ T lit_axpy(Cf c, T x, T y) {
     A::cfma(c, x, y);
     return y;
   }
-  static __device__ __forceinline__ T axpy(double c, T x, T y) { return axpy(cf_of(c), x, y); }
-  static __device__ __forceinline__ T sub(T a, T b) { return A::add(a, A::neg(b)); }
 
   // nodal values -> values at the Gauss points
-  static __device__ __forceinline__ void interp(const T (&u)[N], T (&v)[N]) {
+  __device__ __forceinline__ void interp(const T (&u)[N], T (&v)[N]) const {
     if constexpr (A::kDW || K == 1) {
       dense([](int a, int j) { return cS<K>(a, j); }, u, v);
     } else if constexpr (K == 2) {
-      const T s = A::add(u[0], u[2]), d = sub(u[2], u[0]);
-      const T e = axpy(0.3, s, A::cmul(cf_of(0.4), u[1]));
-      v[0] = axpy(-kB2(), d, e);
+      const T s = add(u[0], u[2]), d = sub(u[2], u[0]);
+      const T e = axpy<kA2>(s, scale<kM2>(u[1]));
+      v[0] = axmy<kB2>(d, e);
       v[1] = u[1];
-      v[2] = axpy(kB2(), d, e);
+      v[2] = axpy<kB2>(d, e);
     } else {
       T eo, ei;
       cubic(u, v, eo, ei);
     }
   }
-  // values at the Gauss points -> derivatives there, in units of deriv_scale
-  static __device__ __forceinline__ void deriv(const T (&v)[N], T (&g)[N]) {
+  // values at the Gauss points -> derivatives there, in the scaled unit
+  __device__ __forceinline__ void deriv(const T (&v)[N], T (&g)[N]) const {
     if constexpr (K == 1) {
-      g[0] = g[1] = A::fin(axpy(cD<1>(1, 1), v[1], A::cmul(cD<1>(1, 0), v[0])));
+      g[0] = g[1] = A::fin(lit_axpy(cD<1>(1, 1), v[1], A::cmul(cD<1>(1, 0), v[0])));
     } else if constexpr (K == 2) {
       const T m = sub(v[2], v[0]), a = sub(v[2], v[1]);
-      const T p = axpy(4.0, a, A::neg(m));
-      g[0] = A::fin(axpy(2.0, m, A::neg(p)));
+      const T p = axpy<kFour>(a, A::neg(m));
+      g[0] = A::fin(axpy<kTwo>(m, A::neg(p)));
       g[1] = A::fin(m);
       g[2] = A::fin(p);
     } else {
-      const T q = sub(A::add(v[0], v[3]), A::add(v[1], v[2]));
+      const T q = sub(add(v[0], v[3]), add(v[1], v[2]));
       cubic_deriv(sub(v[3], v[0]), sub(v[2], v[1]), q, g);
     }
   }
   // both at once (v as interp, g as deriv of v)
-  static __device__ __forceinline__ void interp_deriv(const T (&u)[N], T (&v)[N], T (&g)[N]) {
+  __device__ __forceinline__ void interp_deriv(const T (&u)[N], T (&v)[N], T (&g)[N]) const {
     if constexpr (!A::kDW && K == 2) {
-      const T s = A::add(u[0], u[2]), d = sub(u[2], u[0]);
-      const T t = axpy(-2.0, u[1], s);
-      const T e = axpy(0.3, t, u[1]), m = A::cmul(cf_of(2.0 * kB2()), d);
-      v[0] = axpy(-0.5, m, e);
+      const T s = add(u[0], u[2]), d = sub(u[2], u[0]);
+      const T t = axmy<kTwo>(u[1], s);
+      const T e = axpy<kA2>(t, u[1]);
+      v[0] = axmy<kB2>(d, e);
       v[1] = u[1];
-      v[2] = axpy(0.5, m, e);
-      g[0] = axpy(-1.2, t, m);
+      v[2] = axpy<kB2>(d, e);
+      const T m = sub(v[2], v[0]);
+      g[0] = axmy<kG2>(t, m);
       g[1] = m;
-      g[2] = axpy(1.2, t, m);
+      g[2] = axpy<kG2>(t, m);
     } else if constexpr (!A::kDW && K == 3) {
       T eo, ei;
       cubic(u, v, eo, ei);
       const T q = sub(eo, ei);
-      cubic_deriv(sub(v[3], v[0]), sub(v[2], v[1]), A::add(q, q), g);
+      cubic_deriv(sub(v[3], v[0]), sub(v[2], v[1]), add(q, q), g);
     } else {
       interp(u, v);
       deriv(v, g);
     }
   }
   // r += transpose of deriv applied to g (sums still to be finished)
-  static __device__ __forceinline__ void deriv_t(const T (&g)[N], T (&r)[N]) {
+  __device__ __forceinline__ void deriv_t(const T (&g)[N], T (&r)[N]) const {
     if constexpr (K == 1) {
-      const T G = A::add(g[0], g[1]);
-      r[0] = axpy(cD<1>(0, 0), G, r[0]);
-      r[1] = axpy(cD<1>(0, 1), G, r[1]);
+      const T G = add(g[0], g[1]);
+      r[0] = lit_axpy(cD<1>(0, 0), G, r[0]);
+      r[1] = lit_axpy(cD<1>(0, 1), G, r[1]);
     } else if constexpr (K == 2) {
       const T P = sub(g[2], g[0]);
-      const T B = sub(axpy(2.0, g[0], g[1]), P);   // the odd part: -B on one end, B + 4 P on the other
+      const T B = sub(axpy<kTwo>(g[0], g[1]), P);   // the odd part: -B on one end, B + 4 P on the other
       r[0] = sub(r[0], B);
-      r[1] = axpy(-4.0, P, r[1]);
-      r[2] = axpy(4.0, P, A::add(r[2], B));
-    } else {
+      r[1] = axmy<kFour>(P, r[1]);
+      r[2] = axpy<kFour>(P, add(r[2], B));
+    } else if constexpr (A::kDW) {
 #pragma unroll
       for (int a = 0; a < N; ++a)
 #pragma unroll
-        for (int j = 0; j < N; ++j) r[a] = axpy(RefShape<3>::D(j, a) / deriv_scale<3>(), g[j], r[a]);
+        for (int j = 0; j < N; ++j) r[a] = lit_axpy(cf_of(deriv_const(j, a)), g[j], r[a]);
+    } else {
+      const T Go = add(g[0], g[3]), Gi = add(g[1], g[2]), Ho = sub(g[3], g[0]), Hi = sub(g[2], g[1]);
+      const T Q = axpy<kQo>(Ho, scale<kQi>(Hi));
+      const T X = axpy<kAi>(Gi, Go), Y = axpy<kBi>(Gi, scale<kBo>(Go));
+      r[0] = sub(add(r[0], Q), X);
+      r[1] = sub(sub(r[1], Q), Y);
+      r[2] = add(sub(r[2], Q), Y);
+      r[3] = add(add(r[3], Q), X);
     }
   }
   // transpose of interp
-  static __device__ __forceinline__ void interp_t(const T (&r)[N], T (&n)[N]) {
+  __device__ __forceinline__ void interp_t(const T (&r)[N], T (&n)[N]) const {
     if constexpr (A::kDW || K == 1) {
       dense([](int a, int j) { return cS<K>(j, a); }, r, n);
     } else if constexpr (K == 2) {
-      quad_t(A::add(r[0], r[2]), sub(r[2], r[0]), r[1], n);
+      quad_t(add(r[0], r[2]), sub(r[2], r[0]), r[1], n);
     } else {
-      cubic_t(A::add(r[0], r[3]), A::add(r[1], r[2]), sub(r[3], r[0]), sub(r[2], r[1]), n);
+      cubic_t(add(r[0], r[3]), add(r[1], r[2]), sub(r[3], r[0]), sub(r[2], r[1]), n);
     }
   }
   // n = transpose of interp applied to (r + transpose of deriv applied to g)
-  static __device__ __forceinline__ void interp_deriv_t(T (&r)[N], const T (&g)[N], T (&n)[N]) {
+  __device__ __forceinline__ void interp_deriv_t(T (&r)[N], const T (&g)[N], T (&n)[N]) const {
     if constexpr (!A::kDW && K == 2) {
-      const T P = sub(g[2], g[0]), S = A::add(A::add(g[0], g[2]), g[1]);
-      quad_t(axpy(4.0, P, A::add(r[0], r[2])), axpy(2.0, S, sub(r[2], r[0])), axpy(-4.0, P, r[1]), n);
+      const T P = sub(g[2], g[0]), S = add(add(g[0], g[2]), g[1]);
+      quad_t(axpy<kFour>(P, add(r[0], r[2])), axpy<kTwo>(S, sub(r[2], r[0])), axmy<kFour>(P, r[1]), n);
     } else if constexpr (!A::kDW && K == 3) {
-      const T Go = A::add(g[0], g[3]), Gi = A::add(g[1], g[2]), Ho = sub(g[3], g[0]), Hi = sub(g[2], g[1]);
-      const T Q = axpy(2.0 * kQo(), Ho, A::cmul(cf_of(2.0 * kQi()), Hi));
-      const T so = A::add(A::add(r[0], r[3]), Q), si = sub(A::add(r[1], r[2]), Q);
-      const T dO = axpy(2.0 * kAi(), Gi, axpy(2.0, Go, sub(r[3], r[0])));
-      const T dI = axpy(2.0 * kBi(), Gi, axpy(2.0 * kBo(), Go, sub(r[2], r[1])));
+      const T Go = add(g[0], g[3]), Gi = add(g[1], g[2]), Ho = sub(g[3], g[0]), Hi = sub(g[2], g[1]);
+      const T Q = axpy<kQo2>(Ho, scale<kQi2>(Hi));
+      const T so = add(add(r[0], r[3]), Q), si = sub(add(r[1], r[2]), Q);
+      const T dO = axpy<kAi2>(Gi, axpy<kTwo>(Go, sub(r[3], r[0])));
+      const T dI = axpy<kBi2>(Gi, axpy<kBo2>(Go, sub(r[2], r[1])));
       cubic_t(so, si, dO, dI, n);
     } else {
       deriv_t(g, r);
@@ -202,48 +274,43 @@ struct Line {
   }
 
  private:
-  // Q2: half the difference of the end functions at the outer Gauss point (sqrt(3/5) / 2);
-  // their mean there is 0.3, the middle function 0.4
-  static __host__ __device__ constexpr double kB2() { return 0.5 * (RefShape<2>::S(2, 2) - RefShape<2>::S(2, 0)); }
-  static __device__ __forceinline__ void quad_t(T s, T o, T r1, T (&n)[N]) {
-    const T t = A::cmul(cf_of(0.3), s);
-    n[0] = axpy(-kB2(), o, t);
-    n[1] = axpy(0.4, s, r1);
-    n[2] = axpy(kB2(), o, t);
+  // Q3: weight of value a in the derivative at point j, from the parts
+  static __host__ __device__ constexpr double deriv_const(int j, int a) {
+    const bool inner = j == 1 || j == 2, in_a = a == 1 || a == 2;
+    const double odd = inner ? line_const<3>(in_a ? kBi : kAi) : (in_a ? line_const<3>(kBo) : 1.0);
+    const double even = line_const<3>(inner ? kQi : kQo);
+    return (a >= 2 ? odd : -odd) + ((j >= 2) != in_a ? even : -even);
   }
-  // Q3: even (E) and odd (C) parts of the end (0) and inner (1) basis functions at the outer (o) and
-  // inner (i) Gauss points, and the derivative's weights on (v3 - v0), (v2 - v1) and (v0 + v3) - (v1 + v2)
-  static __host__ __device__ constexpr double sE(int q, int n) { return 0.5 * (RefShape<3>::S(q, n) + RefShape<3>::S(q, 3 - n)); }
-  static __host__ __device__ constexpr double sC(int q, int n) { return 0.5 * (RefShape<3>::S(q, n) - RefShape<3>::S(q, 3 - n)); }
-  static __host__ __device__ constexpr double kQo() { return 0.5 * (RefShape<3>::D(3, 3) + RefShape<3>::D(3, 0)) / deriv_scale<3>(); }
-  static __host__ __device__ constexpr double kQi() { return 0.5 * (RefShape<3>::D(2, 3) + RefShape<3>::D(2, 0)) / deriv_scale<3>(); }
-  static __host__ __device__ constexpr double kAi() { return 0.5 * (RefShape<3>::D(2, 3) - RefShape<3>::D(2, 0)) / deriv_scale<3>(); }
-  static __host__ __device__ constexpr double kBo() { return 0.5 * (RefShape<3>::D(3, 2) - RefShape<3>::D(3, 1)) / deriv_scale<3>(); }
-  static __host__ __device__ constexpr double kBi() { return 0.5 * (RefShape<3>::D(2, 2) - RefShape<3>::D(2, 1)) / deriv_scale<3>(); }
-  static __device__ __forceinline__ void cubic(const T (&u)[N], T (&v)[N], T& eo, T& ei) {
-    const T s0 = A::add(u[0], u[3]), s1 = A::add(u[1], u[2]), d0 = sub(u[3], u[0]), d1 = sub(u[2], u[1]);
-    eo = axpy(sE(3, 2), s1, A::cmul(cf_of(sE(3, 3)), s0));
-    ei = axpy(sE(2, 2), s1, A::cmul(cf_of(sE(2, 3)), s0));
-    const T wo = axpy(sC(3, 2) / sC(3, 3), d1, d0), wi = axpy(sC(2, 3) / sC(2, 2), d0, d1);
-    v[0] = axpy(-sC(3, 3), wo, eo);
-    v[1] = axpy(-sC(2, 2), wi, ei);
-    v[2] = axpy(sC(2, 2), wi, ei);
-    v[3] = axpy(sC(3, 3), wo, eo);
+  __device__ __forceinline__ void quad_t(T s, T o, T r1, T (&n)[N]) const {
+    const T t = scale<kA2>(s);
+    n[0] = axmy<kB2>(o, t);
+    n[1] = axpy<kM2>(s, r1);
+    n[2] = axpy<kB2>(o, t);
   }
-  static __device__ __forceinline__ void cubic_deriv(T d0, T d1, T q, T (&g)[N]) {
-    const T eo = axpy(kBo(), d1, d0), ei = axpy(kBi(), d1, A::cmul(cf_of(kAi()), d0));
-    g[0] = A::fin(axpy(-kQo(), q, eo));
-    g[1] = A::fin(axpy(-kQi(), q, ei));
-    g[2] = A::fin(axpy(kQi(), q, ei));
-    g[3] = A::fin(axpy(kQo(), q, eo));
+  __device__ __forceinline__ void cubic(const T (&u)[N], T (&v)[N], T& eo, T& ei) const {
+    const T s0 = add(u[0], u[3]), s1 = add(u[1], u[2]), d0 = sub(u[3], u[0]), d1 = sub(u[2], u[1]);
+    eo = axpy<kEo1>(s1, scale<kEo0>(s0));
+    ei = axpy<kEi1>(s1, scale<kEi0>(s0));
+    const T wo = axpy<kRo>(d1, d0), wi = axpy<kRi>(d0, d1);
+    v[0] = axmy<kCo>(wo, eo);
+    v[1] = axmy<kCi>(wi, ei);
+    v[2] = axpy<kCi>(wi, ei);
+    v[3] = axpy<kCo>(wo, eo);
   }
-  static __device__ __forceinline__ void cubic_t(T so, T si, T dO, T dI, T (&n)[N]) {
-    const T n0 = axpy(sE(2, 3), si, A::cmul(cf_of(sE(3, 3)), so)), n1 = axpy(sE(2, 2), si, A::cmul(cf_of(sE(3, 2)), so));
-    const T x0 = axpy(sC(2, 3) / sC(3, 3), dI, dO), x1 = axpy(sC(3, 2) / sC(2, 2), dO, dI);
-    n[0] = axpy(-sC(3, 3), x0, n0);
-    n[1] = axpy(-sC(2, 2), x1, n1);
-    n[2] = axpy(sC(2, 2), x1, n1);
-    n[3] = axpy(sC(3, 3), x0, n0);
+  __device__ __forceinline__ void cubic_deriv(T d0, T d1, T q, T (&g)[N]) const {
+    const T eo = axpy<kBo>(d1, d0), ei = axpy<kBi>(d1, scale<kAi>(d0));
+    g[0] = A::fin(axmy<kQo>(q, eo));
+    g[1] = A::fin(axmy<kQi>(q, ei));
+    g[2] = A::fin(axpy<kQi>(q, ei));
+    g[3] = A::fin(axpy<kQo>(q, eo));
+  }
+  __device__ __forceinline__ void cubic_t(T so, T si, T dO, T dI, T (&n)[N]) const {
+    const T n0 = axpy<kEi0>(si, scale<kEo0>(so)), n1 = axpy<kEi1>(si, scale<kEo1>(so));
+    const T x0 = axpy<kTo>(dI, dO), x1 = axpy<kTi>(dO, dI);
+    n[0] = axmy<kCo>(x0, n0);
+    n[1] = axmy<kCi>(x1, n1);
+    n[2] = axpy<kCi>(x1, n1);
+    n[3] = axpy<kCo>(x0, n0);
   }
 };
 
@@ -260,13 +327,12 @@ __host__ __device__ constexpr int line_first(int d, int i) {
 
 // --------------------------------------------------------------- phase 1
 // Nodal values u (lexicographic, x fastest) -> values and reference gradients
-// (in units of deriv_scale) at the tensor Gauss points: x, then y (, then z)
+// (in that unit) at the tensor Gauss points: x, then y (, then z)
 // interpolation in place, the last direction with its derivative; the other
 // derivatives by collocation.  put(comp * NQD + point, value) stores them.
 template <class A, int DIM, int K, class Put>
-__device__ __forceinline__ void forward_cell(typename A::T* u, Put put) {
+__device__ __forceinline__ void forward_cell(const Line<A, K>& L, typename A::T* u, Put put) {
   using T = typename A::T;
-  using L = Line<A, K>;
   constexpr int N = K + 1, NQD = Shape<DIM, K>::NQD, NL = NQD / N;
   T in[N], v[N], g[N];
 #pragma unroll
@@ -278,9 +344,9 @@ __device__ __forceinline__ void forward_cell(typename A::T* u, Put put) {
 #pragma unroll
       for (int j = 0; j < N; ++j) in[j] = u[o + j * st];
       if (d + 1 < DIM) {
-        L::interp(in, v);
+        L.interp(in, v);
       } else {
-        L::interp_deriv(in, v, g);
+        L.interp_deriv(in, v, g);
 #pragma unroll
         for (int j = 0; j < N; ++j) put((1 + d) * NQD + o + j * st, g[j]);
       }
@@ -299,7 +365,7 @@ __device__ __forceinline__ void forward_cell(typename A::T* u, Put put) {
       const int o = line_first<N>(d, i);
 #pragma unroll
       for (int j = 0; j < N; ++j) in[j] = u[o + j * st];
-      L::deriv(in, g);
+      L.deriv(in, g);
 #pragma unroll
       for (int j = 0; j < N; ++j) put((1 + d) * NQD + o + j * st, g[j]);
     }
@@ -310,9 +376,8 @@ __device__ __forceinline__ void forward_cell(typename A::T* u, Put put) {
 // Point values and reference-gradient coefficients (get(comp * NQD + point))
 // -> nodal contributions r: the transpose of forward_cell.
 template <class A, int DIM, int K, class Get>
-__device__ __forceinline__ void backward_cell(Get get, typename A::T* r) {
+__device__ __forceinline__ void backward_cell(const Line<A, K>& L, Get get, typename A::T* r) {
   using T = typename A::T;
-  using L = Line<A, K>;
   constexpr int N = K + 1, NQD = Shape<DIM, K>::NQD, NL = NQD / N;
   T in[N], g[N], out[N];
 #pragma unroll
@@ -328,7 +393,7 @@ __device__ __forceinline__ void backward_cell(Get get, typename A::T* r) {
         in[j] = r[o + j * st];
         g[j] = get((1 + d) * NQD + o + j * st);
       }
-      L::deriv_t(g, in);
+      L.deriv_t(g, in);
 #pragma unroll
       for (int j = 0; j < N; ++j) r[o + j * st] = in[j];
     }
@@ -344,9 +409,9 @@ __device__ __forceinline__ void backward_cell(Get get, typename A::T* r) {
       if (d + 1 == DIM) {
 #pragma unroll
         for (int j = 0; j < N; ++j) g[j] = get((1 + d) * NQD + o + j * st);
-        L::interp_deriv_t(in, g, out);
+        L.interp_deriv_t(in, g, out);
       } else {
-        L::interp_t(in, out);
+        L.interp_t(in, out);
       }
 #pragma unroll
       for (int j = 0; j < N; ++j) r[o + j * st] = out[j];
@@ -381,7 +446,7 @@ struct ChunkBounds {
 // The persistent chunk kernel (design notes in sg_apply.cu).
 template <class A, int DIM, int K, int NT>
 __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<DIM, K, NT>::blocks)
-    sg_apply_chunk_kernel(const ApplyParams p) {
+    sg_apply_chunk_kernel(const __grid_constant__ ApplyParams p) {
   using T = typename A::T;
   using Sh = Shape<DIM, K>;
   constexpr int NQD = Sh::NQD, NKD = Sh::NKD, NC = Sh::NC, N = Sh::N;
@@ -393,6 +458,9 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int n_xi = p.n_xi, V = n_xi * NT, C = p.chunk;
+  __shared__ double s_lk[kLineConsts];   // an array of its own: stores to the values cannot alias it
+  if (std::is_same<A, F64>::value && tid < kLineConsts) s_lk[tid] = p.lk[tid];   // visible after the first barrier
+  const Line<A, K> L(s_lk);
 
   const bool premul = p.premul != 0;
   const int rows = premul ? p.n_pairs : p.n_terms;              // coefficient rows per cell
@@ -401,7 +469,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
   T* Amq = Cs + (size_t)C * rows * NQD;                         // [NQD][NT][NT]
   T* Tb = Amq + NQD * NT * NT;                                  // [NT]
   T* Rt = Tb + NT;                                              // [3] (h_0/h_d)^2
-  T* Gv = Rt + 3;                                               // G per pair (premul) or per entry
+  T* Gv = Rt + 3;                                               // G per entry (unused with premul)
   // the packed coupling entries follow at a 16-byte boundary
   CoupleEntry* Ge = reinterpret_cast<CoupleEntry*>(
       (reinterpret_cast<uintptr_t>(Gv + (premul ? p.n_pairs : p.nnz)) + 15) & ~static_cast<uintptr_t>(15));
@@ -411,12 +479,9 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
   int* Nd = Pt + (premul ? p.n_pairs : 0);                      // [C][NKD] node of y / x, -1 on the boundary
 
   if (premul) {
-    for (int k = tid; k < p.n_pairs; k += nthr) {
-      Gv[k] = A::in(p.pair_val[k] * grad_weight<K>());
-      Pt[k] = p.pair_term[k];
-    }
+    for (int k = tid; k < p.n_pairs; k += nthr) Pt[k] = p.pair_term[k];
   } else {
-    for (int e = tid; e < p.nnz; e += nthr) Gv[e] = A::in(p.g_val[e] * grad_weight<K>());
+    for (int e = tid; e < p.nnz; e += nthr) Gv[e] = A::in(p.g_val[e]);
   }
   for (int e = tid; e < p.nnz; e += nthr) {
     CoupleEntry ce;
@@ -435,7 +500,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
   for (int e = tid; e <= n_xi; e += nthr) Gr[e] = p.g_row[e];
   for (int e = tid; e < n_xi; e += nthr) Pm[e] = p.perm[e];
   for (int e = tid; e < NQD * NT * NT; e += nthr) Amq[e] = A::in(p.amq[e]);
-  if (tid < NT) Tb[tid] = A::in(p.tb[tid]);
+  if (tid < NT) Tb[tid] = A::in(p.mode == kApplyResidual ? -p.tb[tid] : p.tb[tid]);
   if (tid < 3) Rt[tid] = A::in(p.ratio[tid]);
 
   const long long c_begin = (long long)blockIdx.x * p.n_cells / gridDim.x;
@@ -453,18 +518,19 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
     {
       const int per_cell = p.n_terms * NQD;
       if (premul) {
-        // G value x a_term(x_q) per (cell, pair, point); the G values carry the
-        // gradients' common factor (grad_weight)
+        // G value x a_term(x_q) per (cell, pair, point), multiplied in FP64
+        // and converted once; pair_w carries the gradients' weight
         const int per_row = rows * NQD;
         for (int idx = tid; idx < nc * per_row; idx += nthr) {
           const int c = idx / per_row, r = idx - c * per_row;
           const int k = r / NQD, q = r - k * NQD;
           const long long at = (c0 + c) * per_cell + Pt[k] * NQD + q;
-          if (SG_IN(at, p.n_cells * per_cell, 101)) Cs[idx] = A::fin(A::mul(Gv[k], A::in(p.ctab[at])));
+          if (SG_IN(at, p.n_cells * per_cell, 101)) Cs[idx] = A::in(p.pair_w[k] * p.ctab[at]);
         }
       } else {
         for (int idx = tid; idx < nc * per_cell; idx += nthr)
-          if (SG_IN(c0 * per_cell + idx, p.n_cells * per_cell, 101)) Cs[idx] = A::in(p.ctab[c0 * per_cell + idx]);
+          if (SG_IN(c0 * per_cell + idx, p.n_cells * per_cell, 101))
+            Cs[idx] = A::in(grad_weight<K>() * p.ctab[c0 * per_cell + idx]);
       }
     }
     // the global node of every (cell, local node) of the chunk, once per
@@ -514,7 +580,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
       T u[NKD];
 #pragma unroll
       for (int a = 0; a < NKD; ++a) u[a] = q[a];
-      forward_cell<A, DIM, K>(u, [&](int o, T v) { q[o] = v; });
+      forward_cell<A, DIM, K>(L, u, [&](int o, T v) { q[o] = v; });
     }
     __syncthreads();
     // ---------------------------------------------------------- phase 2
@@ -552,7 +618,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
             const T* am = Amq + q * NT * NT;
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
-              T s = A::mul(am[i * NT], uv[0]);
+              T s = L.mul(am[i * NT], uv[0]);
 #pragma unroll
               for (int j = 1; j < NT; ++j) A::fma(am[i * NT + j], uv[j], s);
               out[kk][i][0] = A::fin(s);
@@ -577,7 +643,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
                   const int ee = -1 - ce.tq;
                   const long long at = (c0 + c) * p.n_terms * NQD + p.g_term[ee] * NQD + q;
                   const double a_q = SG_IN(at, p.n_cells * p.n_terms * NQD, 108) ? p.ctab[at] : 0.0;
-                  couple(A::fin(A::mul(A::in(p.g_val[ee] * grad_weight<K>()), A::in(a_q))), ce.off);
+                  couple(A::fin(A::mul(A::in(p.g_val[ee]), A::in(grad_weight<K>() * a_q))), ce.off);
                 }
               }
             } else {
@@ -590,7 +656,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
             for (int i = 0; i < NT; ++i)
 #pragma unroll
               for (int d = 0; d < DIM; ++d) {
-                if (p.aniso && d > 0) out[kk][i][1 + d] = A::mul(A::fin(out[kk][i][1 + d]), Rt[d]);
+                if (p.aniso && d > 0) out[kk][i][1 + d] = L.mul(A::fin(out[kk][i][1 + d]), Rt[d]);
                 out[kk][i][1 + d] = A::fin(out[kk][i][1 + d]);
               }
           }
@@ -612,7 +678,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
     for (int it = tid; it < nc * V; it += nthr) {
       T* q = Qs + (size_t)it * SLOT;
       T r[NKD];
-      backward_cell<A, DIM, K>([&](int o) { return q[o]; }, r);
+      backward_cell<A, DIM, K>(L, [&](int o) { return q[o]; }, r);
 #pragma unroll
       for (int a = 0; a < NKD; ++a) q[a] = r[a];
     }
@@ -625,8 +691,7 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
         const int v = j / NKD, a = j - v * NKD;
         const int node = nd[a];
         if (node >= 0 && SG_IN((long long)v * p.n_x + node, (long long)V * p.n_x, 107)) {
-          T val = A::mul(Tb[v % NT], qc[(size_t)v * SLOT + a]);
-          if (p.mode == kApplyResidual) val = A::neg(val);
+          T val = L.mul(Tb[v % NT], qc[(size_t)v * SLOT + a]);
           A::add_out(yout + (long long)v * p.n_x + node, val);
         }
       }

@@ -43,13 +43,20 @@ struct DiagArgs {
   int cells[3], nn[3];
   T ratio[3];
   T tb[kMaxNT];             // sign * tau Bhat_ii
+  double lk[kLineConsts];   // constants of the 1D passes
   T amq[kMaxAmq];           // [point][i][j] w_q |J| T[i][j] / (tau Bhat_ii)
 };
 
 template <class A, int DIM, int K, int NT>
 __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_constant__ DiagArgs<typename A::T> p) {
   using T = typename A::T;
-  using L = Line<A, K>;
+  __shared__ double s_lk[kLineConsts];
+  if (std::is_same<A, F64>::value) {
+    const int t = threadIdx.y * 32 + threadIdx.x;
+    if (t < kLineConsts) s_lk[t] = p.lk[t];
+    __syncthreads();
+  }
+  const Line<A, K> L(s_lk);
   constexpr int N = K + 1, NQD = Shape<DIM, K>::NQD, NL = NQD / N;
   const int lane = threadIdx.x, row = blockIdx.y * kDiagRows + threadIdx.y;
   if (row >= p.rows) return;                                  // whole warps
@@ -103,7 +110,7 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
         const int o = line_first<N>(d, l), st = line_stride<N>(d);
 #pragma unroll
         for (int j = 0; j < N; ++j) in[j] = v[i][o + j * st];
-        L::interp(in, out);
+        L.interp(in, out);
 #pragma unroll
         for (int j = 0; j < N; ++j) v[i][o + j * st] = out[j];
       }
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
     T r[NQD];
 #pragma unroll
     for (int q = 0; q < NQD; ++q) {
-      T s = A::mul(p.amq[(q * NT + i) * NT], v[0][q]);
+      T s = L.mul(p.amq[(q * NT + i) * NT], v[0][q]);
 #pragma unroll
       for (int j = 1; j < NT; ++j) A::fma(p.amq[(q * NT + i) * NT + j], v[j][q], s);
       r[q] = s;
@@ -132,20 +139,20 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
         if (!p.mass_only) {
 #pragma unroll
           for (int j = 0; j < N; ++j) in[j] = v[i][o + j * st];
-          L::deriv(in, g);
+          L.deriv(in, g);
 #pragma unroll
-          for (int j = 0; j < N; ++j) g[j] = A::mul(g[j], c[o + j * st]);
+          for (int j = 0; j < N; ++j) g[j] = L.mul(g[j], c[o + j * st]);
           if (dd > 0 && p.aniso) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) g[j] = A::mul(g[j], p.ratio[dd]);
+            for (int j = 0; j < N; ++j) g[j] = L.mul(g[j], p.ratio[dd]);
           }
           if (dd + 1 < DIM) {
-            L::deriv_t(g, rl);
+            L.deriv_t(g, rl);
           } else {
-            L::interp_deriv_t(rl, g, out);
+            L.interp_deriv_t(rl, g, out);
           }
         } else if (dd + 1 == DIM) {
-          L::interp_t(rl, out);
+          L.interp_t(rl, out);
         }
 #pragma unroll
         for (int j = 0; j < N; ++j) r[o + j * st] = dd + 1 < DIM ? rl[j] : out[j];
@@ -159,7 +166,7 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
         const int o = line_first<N>(dd, l);
 #pragma unroll
         for (int j = 0; j < N; ++j) in[j] = r[o + j * st];
-        L::interp_t(in, out);
+        L.interp_t(in, out);
 #pragma unroll
         for (int j = 0; j < N; ++j) r[o + j * st] = out[j];
       }
@@ -168,12 +175,12 @@ __global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_consta
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
       const T left = __shfl_up_sync(0xffffffffu, r[l * N + K], 1);
-      if (take) r[l * N] = A::add(r[l * N], left);
+      if (take) r[l * N] = L.add(r[l * N], left);
     }
 #pragma unroll
     for (int a = 0; a < NQD; ++a)
       if (inner(a) && !(a % N == K && give) && SG_IN((v0 + i) * p.n_x + offset(a), n_vec, 702))
-        A::add_out(dst + offset(a), A::mul(p.tb[i], r[a]));
+        A::add_out(dst + offset(a), L.mul(p.tb[i], r[a]));
   }
 }
 
@@ -210,6 +217,7 @@ cudaError_t launch(int dim, int k, int nt, const DiagParams& q, cudaStream_t s) 
     p.ratio[d] = (T)q.ratio[d];
     p.aniso |= d > 0 && d < dim && q.ratio[d] != 1.0;
   }
+  fill_line_consts(k, p.lk);
   const int nq = k + 1, nqd = dim == 2 ? nq * nq : nq * nq * nq;
   for (int i = 0; i < nt; ++i) p.tb[i] = (T)(q.sign * q.tb[i]);
   for (int i = 0; i < nqd * nt * nt; ++i) p.amq[i] = (T)q.amq[i];

@@ -17,6 +17,7 @@ constexpr int kMaxNQ = kMaxK + 1; // Gauss points per direction
 constexpr int kMaxNT = 4;         // largest number of time nodes (dG(3))
 constexpr int kMaxQD = 64;        // largest tensor Gauss rule per cell (4^3)
 constexpr int kMaxAmq = 256;      // largest (points x time nodes^2) coupling table
+constexpr int kLineConsts = 24;   // constants of the 1D passes (line_const)
 constexpr int kMaxPairs = 32;     // largest number of distinct (term, G value) pairs pre-multiplied
 
 // ---------------------------------------------------------------- host maths
@@ -108,6 +109,7 @@ struct ApplyParams {
   double ratio[3];        // (h_0 / h_d)^2
   double amq[kMaxAmq];    // [q][i][j] w_q |J| A_t[i][j] / (tau Bhat_ii) (A_t^T for the transpose)
   double tb[kMaxNT];      // tau Bhat_ii
+  double lk[kLineConsts]; // constants of the 1D passes
   const void* b;          // right-hand side of the residual / accumulate modes
   int mode;               // kApplyPlain: y = A x; kApplyResidual: y = b - A x;
                           // kApplyAccumulate: y = b + A x without the Dirichlet identity rows
@@ -120,6 +122,7 @@ struct ApplyParams {
   int n_pairs;
   int pair_term[kMaxPairs];
   double pair_val[kMaxPairs];
+  double pair_w[kMaxPairs];    // pair_val times the weight of the unscaled gradients
 };
 constexpr int kApplyPlain = 0, kApplyResidual = 1, kApplyAccumulate = 2;
 
