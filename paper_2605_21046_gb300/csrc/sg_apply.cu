@@ -203,6 +203,10 @@ sg_status plan_apply_shape(const HostProblem& hp, int chunk, int threads, Launch
   const int kmax = 18 / (hp.n_t * (1 + hp.dim)) < 1 ? 1 : std::min(3, 18 / (hp.n_t * (1 + hp.dim)));
   if (threads <= 0) {
     threads = 256;
+    // double-word is bound by instruction issue with few warps: two CTAs of 384
+    // threads fill the registers where a chunk has work for them (128^2 Q2
+    // M=4 P=4, 3 cells: 589 us against 640 with 256 threads)
+    if (hp.precision == SG_PREC_DW && fa.maxThreadsPerBlock == 384 && chunk * hp.n_xi * hp.n_t >= 384) threads = 384;
     while (threads * kmax < hp.n_xi && threads + 128 <= fa.maxThreadsPerBlock) threads += 128;
   }
   if (threads * kmax < hp.n_xi || threads > fa.maxThreadsPerBlock || threads % 32 || threads < 32) {

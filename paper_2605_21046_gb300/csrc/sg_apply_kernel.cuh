@@ -549,38 +549,54 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
       Nd[i] = interior && SG_IN(node, p.n_x, 102) ? (int)node : -1;
     }
     __syncthreads();
-    // GU values per thread in flight: a batch's loads all issue before its
-    // shared-memory stores
-    constexpr int GU = 4;
-    for (int c = 0; c < nc; ++c) {
-      const int* nd = Nd + c * NKD;
-      T* qc = Qs + (size_t)c * V * SLOT;
-      for (int j0 = tid; j0 < V * NKD; j0 += GU * nthr) {
-        T val[GU];
-        int dst[GU];
+    // FP64 and FP32: the thread of a (cell, vector) loads its nodal values
+    // itself in phase 1.  Double-word, which converts every value it loads,
+    // stages them, spread over all threads.
+    if constexpr (A::kDW) {
+      // GU values per thread in flight: a batch's loads all issue before its
+      // shared-memory stores
+      constexpr int GU = 4;
+      for (int c = 0; c < nc; ++c) {
+        const int* nd = Nd + c * NKD;
+        T* qc = Qs + (size_t)c * V * SLOT;
+        for (int j0 = tid; j0 < V * NKD; j0 += GU * nthr) {
+          T val[GU];
+          int dst[GU];
 #pragma unroll
-        for (int g = 0; g < GU; ++g) {
-          const int j = j0 + g * nthr;
-          const int v = j / NKD, a = j - v * NKD;
-          val[g] = A::zero();
-          dst[g] = j < V * NKD ? v * SLOT + a : -1;
-          const int node = j < V * NKD ? nd[a] : -1;
-          if (node >= 0 && SG_IN((long long)v * p.n_x + node, (long long)V * p.n_x, 103))
-            val[g] = A::in(xin[(long long)v * p.n_x + node]);
+          for (int g = 0; g < GU; ++g) {
+            const int j = j0 + g * nthr;
+            const int v = j / NKD, a = j - v * NKD;
+            val[g] = A::zero();
+            dst[g] = j < V * NKD ? v * SLOT + a : -1;
+            const int node = j < V * NKD ? nd[a] : -1;
+            if (node >= 0 && SG_IN((long long)v * p.n_x + node, (long long)V * p.n_x, 103))
+              val[g] = A::in(xin[(long long)v * p.n_x + node]);
+          }
+#pragma unroll
+          for (int g = 0; g < GU; ++g)
+            if (dst[g] >= 0 && SG_IN((size_t)c * V * SLOT + dst[g], (size_t)C * V * SLOT, 104)) qc[dst[g]] = val[g];
         }
-#pragma unroll
-        for (int g = 0; g < GU; ++g)
-          if (dst[g] >= 0 && SG_IN((size_t)c * V * SLOT + dst[g], (size_t)C * V * SLOT, 104)) qc[dst[g]] = val[g];
       }
+      __syncthreads();
     }
-    __syncthreads();
     // ---------------------------------------------------------- phase 1
     for (int it = tid; it < nc * V; it += nthr) {
       T* q = Qs + (size_t)it * SLOT;
       T u[NKD];
+      if constexpr (A::kDW) {
 #pragma unroll
-      for (int a = 0; a < NKD; ++a) u[a] = q[a];
-      forward_cell<A, DIM, K>(L, u, [&](int o, T v) { q[o] = v; });
+        for (int a = 0; a < NKD; ++a) u[a] = q[a];
+      } else {
+        const int c = it / V, v = it - c * V;
+        const int* nd = Nd + c * NKD;
+        const IO* src = xin + (long long)v * p.n_x;
+#pragma unroll
+        for (int a = 0; a < NKD; ++a) {
+          const int node = nd[a];
+          u[a] = node >= 0 && SG_IN((long long)v * p.n_x + node, (long long)V * p.n_x, 103) ? A::in(src[node]) : A::zero();
+        }
+      }
+      forward_cell<A, DIM, K>(L, u, [&](int o, T val) { q[o] = val; });
     }
     __syncthreads();
     // ---------------------------------------------------------- phase 2
@@ -627,29 +643,89 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
             }
             const T* cq = Cs + (size_t)c * rows * NQD + q;
             const int e_beg = Gr[a], e_end = Gr[a + 1];
-            auto couple = [&](const T w, const int off) {
-              const T* gb = base + off;
-#pragma unroll
-              for (int i = 0; i < NT; ++i)
-#pragma unroll
-                for (int d = 0; d < DIM; ++d) A::fma(w, gb[(size_t)i * SLOT + (1 + d) * NQD], out[kk][i][1 + d]);
-            };
-            if (premul) {
-              for (int e = e_beg; e < e_end; ++e) {
-                const CoupleEntry ce = Ge[e];
-                if (ce.tq >= 0) {
-                  couple(cq[ce.tq], ce.off);
-                } else {
-                  const int ee = -1 - ce.tq;
-                  const long long at = (c0 + c) * p.n_terms * NQD + p.g_term[ee] * NQD + q;
+            if constexpr (A::kDW) {
+              // The first entry starts the sums (a sum costs twice a product) and
+              // the others go two at a time, with the loads of both ahead of their
+              // long arithmetic (128^2 Q2 M=4 P=4 649 -> 626 us).  FP64 takes them
+              // one by one: in pairs, or with the values of one loaded ahead,
+              // 32^3 Q2 went from 2.73 to 2.90 and 3.01 ms.
+              // An entry's weight: the staged product, or G times the staged a_term
+              // (-1 - e marks a pair missing from the pair list: tables from memory).
+              auto weight = [&](int e, const CoupleEntry ce) -> T {
+                if (premul) {
+                  if (ce.tq >= 0) return cq[ce.tq];
+                  const long long at = (c0 + c) * p.n_terms * NQD + p.g_term[e] * NQD + q;
                   const double a_q = SG_IN(at, p.n_cells * p.n_terms * NQD, 108) ? p.ctab[at] : 0.0;
-                  couple(A::fin(A::mul(A::in(p.g_val[ee]), A::in(grad_weight<K>() * a_q))), ce.off);
+                  return A::fin(A::mul(A::in(p.g_val[e]), A::in(grad_weight<K>() * a_q)));
                 }
+                return A::fin(A::mul(Gv[e], cq[ce.tq]));
+              };
+              auto load = [&](const CoupleEntry ce, T (&g)[NT][DIM]) {
+                const T* gb = base + ce.off;
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+#pragma unroll
+                  for (int d = 0; d < DIM; ++d) g[i][d] = gb[(size_t)i * SLOT + (1 + d) * NQD];
+              };
+              auto couple = [&](const T w, const T (&g)[NT][DIM]) {
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+#pragma unroll
+                  for (int d = 0; d < DIM; ++d) A::fma(w, g[i][d], out[kk][i][1 + d]);
+              };
+              int e = e_beg;
+              if (e < e_end) {
+                const CoupleEntry ce = Ge[e];
+                const T w = weight(e, ce);
+                T g[NT][DIM];
+                load(ce, g);
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+#pragma unroll
+                  for (int d = 0; d < DIM; ++d) out[kk][i][1 + d] = A::mul(w, g[i][d]);
+                ++e;
+              }
+              for (; e + 1 < e_end; e += 2) {
+                const CoupleEntry ce0 = Ge[e], ce1 = Ge[e + 1];
+                const T w0 = weight(e, ce0), w1 = weight(e + 1, ce1);
+                T g0[NT][DIM], g1[NT][DIM];
+                load(ce0, g0);
+                load(ce1, g1);
+                couple(w0, g0);
+                couple(w1, g1);
+              }
+              if (e < e_end) {
+                const CoupleEntry ce = Ge[e];
+                const T w = weight(e, ce);
+                T g[NT][DIM];
+                load(ce, g);
+                couple(w, g);
               }
             } else {
-              for (int e = e_beg; e < e_end; ++e) {
-                const CoupleEntry ce = Ge[e];
-                couple(A::fin(A::mul(Gv[e], cq[ce.tq])), ce.off);
+              auto couple = [&](const T w, const int off) {
+                const T* gb = base + off;
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+#pragma unroll
+                  for (int d = 0; d < DIM; ++d) A::fma(w, gb[(size_t)i * SLOT + (1 + d) * NQD], out[kk][i][1 + d]);
+              };
+              if (premul) {
+                for (int e = e_beg; e < e_end; ++e) {
+                  const CoupleEntry ce = Ge[e];
+                  if (ce.tq >= 0) {
+                    couple(cq[ce.tq], ce.off);
+                  } else {
+                    const int ee = -1 - ce.tq;
+                    const long long at = (c0 + c) * p.n_terms * NQD + p.g_term[ee] * NQD + q;
+                    const double a_q = SG_IN(at, p.n_cells * p.n_terms * NQD, 108) ? p.ctab[at] : 0.0;
+                    couple(A::fin(A::mul(A::in(p.g_val[ee]), A::in(grad_weight<K>() * a_q))), ce.off);
+                  }
+                }
+              } else {
+                for (int e = e_beg; e < e_end; ++e) {
+                  const CoupleEntry ce = Ge[e];
+                  couple(A::fin(A::mul(Gv[e], cq[ce.tq])), ce.off);
+                }
               }
             }
 #pragma unroll

@@ -139,14 +139,32 @@ struct DW {
     return s;
   }
   __device__ __forceinline__ static T neg(T a) { return {-a.h, -a.l}; }
+  // Normalisation in three additions instead of TwoSum's six: exact when
+  // |l| <= |h|, and also when sums have cancelled h below l, because h is then
+  // a multiple of l's last place (both come from terms of the larger size).
   __device__ __forceinline__ static T fin(T a) {
-    float s, e;
-    two_sum(a.h, a.l, s, e);
-    return {s, e};
+    const float s = __fadd_rn(a.h, a.l);
+    return {s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
   }
+  // One reduction of h + l rounded to double (normalised first, so that |l| is
+  // at most half of h's last place: 2^28 units): l in units of the last place of
+  // h's double pattern is added to the pattern (twice that where h is a power
+  // of two and l points to zero, since the units below it are half as large).
+  // Values whose l could leave the float range (|h| < 2^-101), infinities and
+  // NaN are added in two parts.
   __device__ __forceinline__ static void add_out(double* y, T v) {
-    atomicAdd(y, widen(v.h));
-    if (v.l != 0.0f) atomicAdd(y, widen(v.l));
+    v = fin(v);
+    const unsigned int u = __float_as_uint(v.h), ef = (u >> 23) & 0xffu;
+    if (ef - 26u < 229u) {   // 26 <= ef <= 254
+      const float scaled = __fmul_rn(__fmul_rn(v.l, __uint_as_float((280u - ef) << 23)), 67108864.0f);   // l 2^(153 - ef) 2^26
+      int n = __float2int_rn(scaled);
+      if (u >> 31) n = -n;
+      if ((u & 0x7fffffu) == 0u && n < 0) n *= 2;
+      atomicAdd(y, __longlong_as_double(__double_as_longlong(widen(v.h)) + n));
+    } else {
+      atomicAdd(y, widen(v.h));
+      if (v.l != 0.0f) atomicAdd(y, widen(v.l));
+    }
   }
 };
 
