@@ -257,7 +257,7 @@ sg_status sg_mg_set_coarse_dofs(sg_ctx* ctx, int max_dofs);
  * diagonal coupling table, 1 the diagonal apply, -1 none on the coarsest),
  * Vanka cells per shared-memory chunk (tensor-core sweep: staging buffers),
  * Vanka chaos modes per tile, patch size
- * N_t (k+1)^d, diagonal classes, Vanka kernel (0 FFMA, 1 tensor cores),
+ * N_t (k+1)^d, diagonal classes, Vanka kernel (0 FFMA, 1 tensor cores, 2 registers),
  * reserved 0}.  SG_ERR_ARG without sg_mg_setup or for a level out of range. */
 sg_status sg_mg_level_info(sg_ctx* ctx, int level, int* info);
 
@@ -276,6 +276,9 @@ sg_status sg_mg_setup_times(sg_ctx* ctx, double* total_ms, double* factor_ms, do
  * FFMA sweep, 1 the tensor-core sweep (SG_PREC_BF16 factors, one diagonal
  * class, patches of at most 64 unknowns, at most 80 modes per tile; the
  * transposed V-cycle keeps the FFMA sweep).
+ * 2 is the register sweep (FP32 vectors, 2D patches of at most 18 unknowns;
+ * it has no chunk or tile, and forcing one of those with vanka_kind -1 leaves
+ * it for the FFMA sweep).
  * The results stay the same up to rounding (the variants compute the same
  * V-cycle).  The next sg_vcycle records a new graph.  SG_ERR_ARG /
  * SG_ERR_UNSUPPORTED (nothing changed) when a level cannot take the variant.

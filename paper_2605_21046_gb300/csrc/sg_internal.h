@@ -210,9 +210,10 @@ struct MGLevel {
   bool chunk_ok = false;     // the SG cell kernel has a launch shape for this level
   void* d_inv = nullptr;     // [class][cell][np][pitch] patch inverses (pitch = np rounded up to 8;
                              //  bf16 when MG::bf16), or coarsest [class][n_int][n_int]
+  float* d_inv_col = nullptr;   // [class][entry][cell]: the inverses of the register sweep (null: it does not apply)
   int vanka_chunk = 0;       // cells per Vanka chunk
   int vanka_tile = 0;        // modes per Vanka tile on this level (0: the multigrid's tile)
-  int vanka_kind = 0;        // Vanka sweep: 0 FFMA kernel, 1 tensor-core kernel (bf16 factors)
+  int vanka_kind = 0;        // Vanka sweep: 0 FFMA kernel, 1 tensor-core kernel (bf16 factors), 2 register kernel
   int ffma_chunk = 0, ffma_tile = 0;   // the FFMA sweep's timed choice (kept while the other sweep runs)
   const void* vanka_r = nullptr;       // residual the next sweep reads when not d_r (the first sweep reads b)
   int* d_inner = nullptr;    // coarsest: dof offset (i * n_x + node) of every interior dof
@@ -276,11 +277,11 @@ void mg_free(MG& mg);
 // Per-level choices of a built multigrid: info = {levels, cells, coarsest,
 // residual (0 SG cell kernel, 1 diagonal apply, -1 none), Vanka cells per
 // chunk, Vanka modes per tile, patch size, diagonal classes, Vanka kernel
-// (0 FFMA, 1 tensor cores), 0}.
+// (0 FFMA, 1 tensor cores, 2 registers), 0}.
 sg_status mg_level_info(const MG& mg, int level, int info[10], std::string& msg);
 // Forces the level residual kind (-1 keep, 0 cell kernel, 1 diagonal apply),
 // the Vanka cells per chunk (0 keep), modes per tile (-1 keep, 0 all) and
-// Vanka kernel (-1 keep, 0 FFMA, 1 tensor cores) on one smoothed level (or
+// Vanka kernel (-1 keep, 0 FFMA, 1 tensor cores, 2 registers) on one smoothed level (or
 // every one with level = -1); drops the captured graphs.
 sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int tile, int kind, std::string& msg);
 // The stored inverse of the Vanka patch of (mode alpha's class, cell) on a
@@ -297,6 +298,13 @@ cudaError_t prepare_vanka_tc(int dim, int k, int nt);
 cudaError_t vanka_tc_wait_probe(unsigned int polls, int* status_out);
 cudaError_t launch_vanka_tc(const HostProblem& hp, const float* r, float* x, const void* inv, const int* blk_alpha,
                             int n_blk, int stages, int tile_slots, int* status, float omega, cudaStream_t s);
+// The register Vanka sweep (2D patches of at most 18 unknowns, FP32 vectors;
+// sg_vanka_reg.cu): whether a shape can take it, its copy of the inverses
+// (allocates *out), and one sweep.
+bool vanka_reg_eligible(int dim, int k, int nt);
+cudaError_t vanka_reg_columns(const void* inv, bool bf16, int np, int npp, int n_classes, long long n_cells, float** out);
+cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, const float* inv, const int* blk_cls,
+                             const int* blk_alpha, int n_blk, int n_classes, float omega, int trans, cudaStream_t s);
 // Vanka patch inverses of one multigrid level, assembled and inverted in FP64
 // on the device (Gauss-Jordan, partial pivoting) for every class and cell:
 // out[class][cell][np][npp] as double (out_kind 0), float (1) or bf16 (2).

@@ -624,38 +624,54 @@ __global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferPar
   }
 }
 
-// Coarsest level: x[inner] = inv(C_class) b[inner] for every chaos mode
-// (blockIdx.y) and a block of rows (blockIdx.x); the right-hand side is
-// staged in shared memory.  A warp takes one row of inv (its lanes read the
-// row coalesced and reduce with shuffles); the transposed cycle takes a
-// column per thread (consecutive threads, consecutive columns).
+// Coarsest level: x[inner] = inv(C_class) b[inner] for every chaos mode.  A
+// block takes 8 rows of the inverse (a warp each; columns for the transposed
+// cycle) and the kCoarseModes modes of one mode block, all of one class, whose
+// right-hand sides it stages in shared memory: a row is read once for four
+// modes, coalesced, and reduced with shuffles.  Latency bound (450 unknowns,
+// 35 modes: 10 us with a mode per block).
+constexpr int kCoarseModes = kVankaVB;
+constexpr int kCoarseRows = 8;
+
 template <typename T>
-__global__ void mg_coarse(const T* __restrict__ b, T* __restrict__ x, const T* __restrict__ inv,
-                          const int* __restrict__ cls, const long long* __restrict__ inner, int n_int,
-                          int n_t, long long n_x, int trans) {
+__global__ void __launch_bounds__(32 * kCoarseRows) mg_coarse(const T* __restrict__ b, T* __restrict__ x,
+                                                              const T* __restrict__ inv, const int* __restrict__ blk_cls,
+                                                              const int* __restrict__ blk_alpha,
+                                                              const long long* __restrict__ inner, int n_int, int n_t,
+                                                              long long n_x, int trans) {
   extern __shared__ __align__(16) unsigned char sm[];
-  T* bs = reinterpret_cast<T*>(sm);
-  const int alpha = blockIdx.y;
-  const long long base = (long long)alpha * n_t * n_x;
-  for (int i = threadIdx.x; i < n_int; i += blockDim.x) bs[i] = b[base + inner[i]];
-  __syncthreads();
-  const T* M = inv + (long long)cls[alpha] * n_int * n_int;
-  if (trans) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_int; i += gridDim.x * blockDim.x) {
-      T s = T(0);
-      for (int q = 0; q < n_int; ++q) s += M[(long long)q * n_int + i] * bs[q];
-      x[base + inner[i]] = s;
-    }
-  } else {
-    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * warps + warp; i < n_int; i += gridDim.x * warps) {
-      const T* row = M + (long long)i * n_int;
-      T s = T(0);
-      for (int q = lane; q < n_int; q += 32) s += row[q] * bs[q];
+  T* bs = reinterpret_cast<T*>(sm);                            // [mode][n_int]
+  const int blk = blockIdx.y;
+  long long base[kCoarseModes];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) x[base + inner[i]] = s;
-    }
+  for (int u = 0; u < kCoarseModes; ++u) {
+    const int m = __ldg(blk_alpha + blk * kCoarseModes + u);
+    base[u] = m < 0 ? -1 : (long long)m * n_t * n_x;
+  }
+  for (int i = threadIdx.x; i < n_int; i += blockDim.x) {
+    const long long at = __ldg(inner + i);
+#pragma unroll
+    for (int u = 0; u < kCoarseModes; ++u) bs[u * n_int + i] = base[u] >= 0 ? __ldg(b + base[u] + at) : T(0);
+  }
+  __syncthreads();
+  const T* M = inv + (long long)__ldg(blk_cls + blk) * n_int * n_int;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * kCoarseRows + warp;
+  if (i >= n_int) return;
+  const T* row = trans ? M + i : M + (long long)i * n_int;
+  const long long step = trans ? n_int : 1;
+  T s[kCoarseModes] = {};
+#pragma unroll 4
+  for (int q = lane; q < n_int; q += 32) {
+    const T w = __ldg(row + q * step);
+#pragma unroll
+    for (int u = 0; u < kCoarseModes; ++u) s[u] = fma(w, bs[u * n_int + q], s[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < kCoarseModes; ++u) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+    if (lane == 0 && base[u] >= 0) x[base[u] + __ldg(inner + i)] = s[u];
   }
 }
 
@@ -1090,6 +1106,10 @@ cudaError_t prepare_vanka(int dim, int k, int nt, bool f32, bool bf16) {
 template <typename T, int DIM, int K, int NT>
 cudaError_t launch_vanka(MG& mg, MGLevel& L, cudaStream_t s, int trans) {
   if constexpr (std::is_same<T, float>::value) {
+    if (L.vanka_kind == 2)
+      return launch_vanka_reg(L.hp, static_cast<const float*>(L.vanka_r ? L.vanka_r : L.d_r), static_cast<float*>(L.d_x),
+                              L.d_inv_col, mg.d_blk_cls, mg.d_blk_alpha, mg.n_blk, mg.n_classes, (float)mg.omega, trans,
+                              s);
     if (mg.bf16 && L.vanka_kind == 1 && !trans) {
       const int tile = L.vanka_tile > 0 ? L.vanka_tile : mg.vanka_tile;
       const float* r = static_cast<const float*>(L.vanka_r ? L.vanka_r : L.d_r);
@@ -1264,12 +1284,10 @@ cudaError_t issue_vcycle(MG& mg, int l, cudaStream_t s, int trans) {
   MGLevel& L = mg.lv[l];
   const int V = L.hp.n_xi * L.hp.n_t;
   if (L.coarsest) {   // x holds the boundary values and 0 inside (restriction, or the start of a one-level hierarchy)
-    const size_t smem = (size_t)L.n_int * sizeof(T);
-    const int gx = trans ? (L.n_int + 255) / 256 : (L.n_int + 7) / 8;   // rows: a warp each (8 a block)
-    mg_coarse<T><<<dim3(gx, L.hp.n_xi), 256, smem, s>>>(static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x),
-                                              static_cast<const T*>(L.d_inv), mg.d_cls,
-                                              reinterpret_cast<const long long*>(L.d_inner), L.n_int, L.hp.n_t, L.hp.n_x,
-                                              trans);
+    const size_t smem = (size_t)kCoarseModes * L.n_int * sizeof(T);
+    mg_coarse<T><<<dim3((L.n_int + kCoarseRows - 1) / kCoarseRows, mg.n_blk), 32 * kCoarseRows, smem, s>>>(
+        static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x), static_cast<const T*>(L.d_inv), mg.d_blk_cls,
+        mg.d_blk_alpha, reinterpret_cast<const long long*>(L.d_inner), L.n_int, L.hp.n_t, L.hp.n_x, trans);
     return cudaGetLastError();
   }
   cudaError_t e;
@@ -1399,7 +1417,7 @@ static cudaError_t tune_vanka(MG& mg) {
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   for (MGLevel& L : mg.lv) {
-    if (L.coarsest || e != cudaSuccess) continue;
+    if (L.coarsest || L.vanka_kind == 2 || e != cudaSuccess) continue;
     const long long n = (long long)L.hp.n_xi * L.hp.n_t * L.hp.n_x;
     if ((e = cudaMemsetAsync(L.d_r, 0, n * vb, mg.stream)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(L.d_x, 0, n * vb, mg.stream)) != cudaSuccess) break;
@@ -1495,7 +1513,7 @@ void mg_free(MG& mg) {
   mg.d_blk_cls = mg.d_blk_alpha = nullptr;
   for (MGLevel& L : mg.lv) {
     cudaFree(L.d_ctab); cudaFree(L.d_grow); cudaFree(L.d_gcol); cudaFree(L.d_gterm); cudaFree(L.d_gval);
-    cudaFree(L.d_perm); cudaFree(L.d_inv); cudaFree(L.d_inner); cudaFree(L.d_coef);
+    cudaFree(L.d_perm); cudaFree(L.d_inv); cudaFree(L.d_inv_col); cudaFree(L.d_inner); cudaFree(L.d_coef);
     cudaFree(L.d_x); cudaFree(L.d_b); cudaFree(L.d_r);
     for (MGLevel::Transfer* t : {&L.down, &L.up}) {
       for (int d = 0; d < 3; ++d) {
@@ -1508,6 +1526,13 @@ void mg_free(MG& mg) {
   mg.lv.clear();
   mg.stream = nullptr;
   mg.d_cls = nullptr;
+}
+
+// Lets the coarse solve stage up to 2048 unknowns of four modes (64 KB in FP64).
+static cudaError_t prepare_coarse(int precision) {
+  const int most = kCoarseModes * 2048 * (int)sizeof(double);
+  return precision == kPrecF32 ? cudaFuncSetAttribute(&mg_coarse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+                               : cudaFuncSetAttribute(&mg_coarse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // Lets the transfer kernels use more than 48 KB of shared memory (rows of
@@ -1729,6 +1754,7 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
         inv.insert(inv.end(), ci.begin(), ci.end());
       }
       if ((e = upload_vec(reinterpret_cast<long long**>(&L.d_inner), inner_dofs)) != cudaSuccess) break;
+      if ((e = prepare_coarse(precision)) != cudaSuccess) break;
       if ((e = upload_values(&L.d_inv, inv, precision)) != cudaSuccess) break;
     }
     // level apply tables (coefficient stays double; vectors use the MG precision)
@@ -1766,6 +1792,13 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       L.ffma_chunk = L.vanka_chunk;
       if ((e = prepare_vanka(L.hp.dim, L.hp.k, L.hp.n_t, precision == kPrecF32, mg.bf16)) != cudaSuccess) break;
       if (mg.bf16 && (e = prepare_vanka_tc(L.hp.dim, L.hp.k, L.hp.n_t)) != cudaSuccess) break;
+      // FP32 vectors and small 2D patches: the register sweep, always the fastest there
+      // (V-cycle with it and with the tuned FFMA or tensor-core sweep: 64^2 Q2, 35 rows 0.115 and 0.158 ms; 128^2 Q2, 70 rows 0.46 and 0.70)
+      if (precision == kPrecF32 && vanka_reg_eligible(L.hp.dim, L.hp.k, L.hp.n_t)) {
+        if ((e = vanka_reg_columns(L.d_inv, mg.bf16, L.np, npp, mg.n_classes, L.hp.n_cells, &L.d_inv_col)) != cudaSuccess)
+          break;
+        L.vanka_kind = 2;
+      }
     }
     if ((e = upload_vec(&L.d_grow, L.hp.g.row)) != cudaSuccess) break;
     if ((e = upload_vec(&L.d_gcol, L.hp.g.col)) != cudaSuccess) break;
@@ -1840,7 +1873,7 @@ sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int 
     msg = "level out of range";
     return SG_ERR_ARG;
   }
-  if (residual_kind < -1 || residual_kind > 1 || chunk < 0 || chunk > 8 || tile < -1 || kind < -1 || kind > 1) {
+  if (residual_kind < -1 || residual_kind > 1 || chunk < 0 || chunk > 8 || tile < -1 || kind < -1 || kind > 2) {
     msg = "variant out of range";
     return SG_ERR_ARG;
   }
@@ -1864,7 +1897,21 @@ sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int 
         msg = "the SG cell kernel has no launch shape on this level";
         return SG_ERR_UNSUPPORTED;
       }
-      const int kd = kind >= 0 ? kind : L.vanka_kind;
+      // the register sweep has no chunk or tile: asking for one asks for the FFMA sweep
+      const int kd = kind >= 0 ? kind : (L.vanka_kind == 2 && (chunk > 0 || tile >= 0) ? 0 : L.vanka_kind);
+      if (kd == 2) {
+        if (!L.d_inv_col) {
+          msg = "the register Vanka sweep needs FP32 vectors and a 2D patch of at most 18 unknowns";
+          return SG_ERR_UNSUPPORTED;
+        }
+        if (pass == 1) {
+          if (residual_kind >= 0) L.use_diag = residual_kind == 1;
+          L.vanka_kind = kd;
+          L.vanka_chunk = L.ffma_chunk;
+          L.vanka_tile = L.ffma_tile;
+        }
+        continue;
+      }
       // "keep" of a sweep that is not running: the FFMA sweep's last chunk and
       // tile, two staging buffers and all modes for the tensor-core sweep
       const int keep = kd == L.vanka_kind ? L.vanka_chunk : (kd == 0 ? L.ffma_chunk : 2);
