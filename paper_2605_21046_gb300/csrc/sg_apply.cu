@@ -309,7 +309,25 @@ cudaError_t launch_apply(const HostProblem& hp, const LaunchShape& ls, const App
   void* f = select_kernel(hp.precision, hp.dim, hp.k, hp.n_t);
   if (!f) return cudaErrorInvalidValue;
   void* args[] = {const_cast<ApplyParams*>(&prm)};
-  cudaError_t e = cudaLaunchKernel(f, dim3(ls.grid), dim3(ls.threads), args, ls.smem, stream);
+  // The cell kernel needs y's start only before its first reduction, so it may
+  // begin while the start pass runs: its tables, gathers and first chunk hide
+  // the pass and the gap between two launches (45x37 Q2 dG(2) 36.9 -> 34.9 us,
+  // 64^2 Q2 149 -> 147; 8x8 Q1 14.4 -> 11.4, where the caller's host time is next).  Inside a capture the kernels are already back to back, and a
+  // plain edge is recorded.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ls.grid);
+  cfg.blockDim = dim3(ls.threads);
+  cfg.dynamicSmemBytes = ls.smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  e = cudaLaunchKernelExC(&cfg, f, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

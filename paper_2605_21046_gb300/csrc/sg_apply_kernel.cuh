@@ -760,6 +760,9 @@ __global__ void __launch_bounds__(ChunkBounds<DIM, K, NT>::threads, ChunkBounds<
     }
     __syncthreads();
     // ---------------------------------------------------------- phase 4
+    // y's start pass may still be running (launch_apply): wait for it before
+    // the first reduction
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int c = 0; c < nc; ++c) {
       const int* nd = Nd + c * NKD;
       const T* qc = Qs + (size_t)c * V * SLOT;

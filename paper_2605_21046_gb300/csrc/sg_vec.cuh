@@ -26,6 +26,7 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) vec_start(const T* b, const T* __restrict__ x, T* y, int op, long long n,
                                                  int nnx, int nny, int nnz) {
   constexpr int G = 4;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a cell kernel that waits before it reduces into y
   const long long n_groups = (n + G - 1) / G;
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
