@@ -47,8 +47,9 @@ struct DiagArgs {
   T amq[kMaxAmq];           // [point][i][j] w_q |J| T[i][j] / (tau Bhat_ii)
 };
 
+// FP32 3D Q2 would take 168 registers; at 128 (no spills) four blocks share an SM.
 template <class A, int DIM, int K, int NT>
-__global__ void __launch_bounds__(32 * kDiagRows) diag_apply(const __grid_constant__ DiagArgs<typename A::T> p) {
+__global__ void __launch_bounds__(32 * kDiagRows, (std::is_same<A, F32>::value && DIM == 3 && K == 2 ? 4 : 0)) diag_apply(const __grid_constant__ DiagArgs<typename A::T> p) {
   using T = typename A::T;
   __shared__ double s_lk[kLineConsts];
   if (std::is_same<A, F64>::value) {

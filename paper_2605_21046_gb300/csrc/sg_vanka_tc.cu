@@ -156,7 +156,7 @@ struct TcUnit {
 };
 
 template <int DIM, int K, int NT>
-__global__ void __launch_bounds__(kTcThreads, 4) mg_vanka_tc(const TcParams p) {
+__global__ void __launch_bounds__(kTcThreads, 5) mg_vanka_tc(const TcParams p) {
   constexpr int N = K + 1;
   constexpr int NKD = DIM == 2 ? N * N : N * N * N;
   constexpr int NP = NT * NKD;
@@ -515,7 +515,8 @@ cudaError_t vanka_tc_wait_probe(unsigned int polls, int* status_out) {
 }
 
 // slots of a tile rounded up to 16: the column pitch of one split term
-static int tc_slot_pitch(int tile_slots) { return (tile_slots + 15) / 16 * 16; }
+// columns of a split term: a multiple of 8, so that both terms make an N of a multiple of 16
+static int tc_slot_pitch(int tile_slots) { return (tile_slots + 7) / 8 * 8; }
 
 size_t vanka_tc_smem(int dim, int k, int nt, int stages, int tile_slots) {
   const int n = k + 1, lyz = dim == 2 ? n : n * n;
@@ -607,7 +608,8 @@ cudaError_t launch_vanka_tc(const HostProblem& hp, const float* r, float* x, con
   p.slp = tc_slot_pitch(sl);
   p.ncols = kTcTerms * p.slp;             // a multiple of 16, at most 160
   p.tmem_cols = 32;
-  while (p.tmem_cols < p.ncols) p.tmem_cols *= 2;
+  // the read-back takes 16 columns at a time, past the last slot where it must
+  while (p.tmem_cols < p.slp + (sl + 15) / 16 * 16) p.tmem_cols *= 2;
   p.n_x = hp.n_x;
   p.n_cells = hp.n_cells;
   p.n_vec_x = (long long)hp.n_xi * hp.n_t * hp.n_x;
