@@ -14,7 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["sg_setup.cpp", "sg_apply.cu", "sg_apply_f64.cu", "sg_apply_dw.cu", "sg_apply_f32.cu", "sg_mg.cu", "sg_vanka_factor.cu", "sg_vanka_tc.cu", "sg_vanka_reg.cu",
+SOURCES = ["sg_setup.cpp", "sg_apply.cu", "sg_apply_f64.cu", "sg_apply_dw.cu", "sg_apply_f32.cu", "sg_mg.cu", "sg_vanka_factor.cu", "sg_vanka_tc.cu", "sg_vanka_reg.cu", "sg_coarse.cu",
            "sg_krylov.cu", "sg_noalloc.cu", "sg_manufactured.cu", "sg_mc.cu", "sg_diag.cu", "sg_adjoint.cu", "sg_api.cu",
            "sg_debug.cu"]
 # the build with device bounds checks (-DSG_DEBUG_BOUNDS): libsg_debug.so

@@ -254,7 +254,6 @@ struct MG {
   double omega = 0.7;
   int n_classes = 0;
   std::vector<int> cls;           // diagonal class of every chaos row
-  int* d_cls = nullptr;
   std::vector<MGLevel> lv;
   cudaStream_t stream = nullptr;
   cudaGraph_t graph_t[2] = {nullptr, nullptr};       // V-cycle of A (0) and of A^T (1)
@@ -298,6 +297,10 @@ cudaError_t prepare_vanka_tc(int dim, int k, int nt);
 cudaError_t vanka_tc_wait_probe(unsigned int polls, int* status_out);
 cudaError_t launch_vanka_tc(const HostProblem& hp, const float* r, float* x, const void* inv, const int* blk_alpha,
                             int n_blk, int stages, int tile_slots, int* status, float omega, cudaStream_t s);
+// The inverse of a dense n x n matrix (host, row major) into `out` (device,
+// values of the precision), by elimination without exchanges (sg_coarse.cu).
+// ok = false where that fails or its check does; out is then undefined.
+cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int precision, void* out, bool& ok);
 // The register Vanka sweep (2D patches of at most 18 unknowns, FP32 vectors;
 // sg_vanka_reg.cu): whether a shape can take it, its copy of the inverses
 // (allocates *out), and one sweep.

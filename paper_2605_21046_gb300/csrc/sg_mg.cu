@@ -807,8 +807,8 @@ bool node_interior(const HostProblem& hp, const int g[3]) {
 // rows for bf16, float and double).
 int vanka_row_pitch(int np) { return (np + 7) / 8 * 8; }
 
-// Coarsest level: dense inverse of the interior block of one class.
-bool coarse_inverse(const HostProblem& hp, const ElementData& e, const std::vector<double>& diag,
+// Coarsest level: the dense interior block of one class.
+void coarse_matrix(const HostProblem& hp, const ElementData& e, const std::vector<double>& diag,
                     const std::vector<long long>& node_of, std::vector<double>& out) {
   const int n = hp.k + 1, nkd = e.nkd, nt = hp.n_t;
   const int nin = (int)node_of.size();
@@ -842,9 +842,7 @@ bool coarse_inverse(const HostProblem& hp, const ElementData& e, const std::vect
           }
       }
   }
-  if (!invert(C, N)) return false;
   out.swap(C);
-  return true;
 }
 
 // 1D interpolation table of one direction between a fine and a coarse level.
@@ -1502,7 +1500,6 @@ void mg_free(MG& mg) {
     mg.graph_t[t] = nullptr;
   }
   if (mg.stream) cudaStreamDestroy(mg.stream);
-  cudaFree(mg.d_cls);
   cudaFree(mg.d_blk_cls);
   cudaFree(mg.d_blk_alpha);
   cudaFree(mg.d_wused);
@@ -1525,7 +1522,6 @@ void mg_free(MG& mg) {
   }
   mg.lv.clear();
   mg.stream = nullptr;
-  mg.d_cls = nullptr;
 }
 
 // Lets the coarse solve stage up to 2048 unknowns of four modes (64 KB in FP64).
@@ -1733,7 +1729,6 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
     L.np = L.hp.n_t * nkd;
     if (L.coarsest) {
       const ElementData ed = element_data(L.hp);
-      std::vector<double> inv;
       std::vector<long long> node_of;
       for (long long m = 0; m < L.hp.n_x; ++m) {
         const int g[3] = {(int)(m % L.hp.nn[0]), (int)((m / L.hp.nn[0]) % L.hp.nn[1]),
@@ -1748,14 +1743,27 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       std::vector<long long> inner_dofs;
       for (int i = 0; i < L.hp.n_t; ++i)
         for (long long m : node_of) inner_dofs.push_back((long long)i * L.hp.n_x + m);
-      for (int c = 0; c < mg.n_classes; ++c) {
+      const size_t vb_c = precision == kPrecF32 ? 4 : 8, n2 = (size_t)L.n_int * L.n_int;
+      if ((e = cudaMalloc(&L.d_inv, mg.n_classes * n2 * vb_c)) != cudaSuccess) break;
+      for (int c = 0; c < mg.n_classes && e == cudaSuccess; ++c) {
         std::vector<double> ci;
-        if (!coarse_inverse(L.hp, ed, class_diag[c], node_of, ci)) { msg = "singular coarse operator"; return SG_ERR_ARG; }
-        inv.insert(inv.end(), ci.begin(), ci.end());
+        void* dst = static_cast<char*>(L.d_inv) + c * n2 * vb_c;
+        bool ok = false;
+        coarse_matrix(L.hp, ed, class_diag[c], node_of, ci);
+        e = coarse_inverse_device(ci, L.n_int, precision, dst, ok);
+        if (ok || e != cudaSuccess) continue;
+        // pivoting elimination on the host
+        if (!invert(ci, L.n_int)) { msg = "singular coarse operator"; return SG_ERR_ARG; }
+        if (precision == kPrecF32) {
+          const std::vector<float> f(ci.begin(), ci.end());
+          e = cudaMemcpy(dst, f.data(), n2 * vb_c, cudaMemcpyHostToDevice);
+        } else {
+          e = cudaMemcpy(dst, ci.data(), n2 * vb_c, cudaMemcpyHostToDevice);
+        }
       }
+      if (e != cudaSuccess) break;
       if ((e = upload_vec(reinterpret_cast<long long**>(&L.d_inner), inner_dofs)) != cudaSuccess) break;
       if ((e = prepare_coarse(precision)) != cudaSuccess) break;
-      if ((e = upload_values(&L.d_inv, inv, precision)) != cudaSuccess) break;
     }
     // level apply tables (coefficient stays double; vectors use the MG precision)
     if ((e = upload_vec(reinterpret_cast<double**>(&L.d_ctab), L.hp.ctab)) != cudaSuccess) break;
@@ -1815,7 +1823,6 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       if ((e = build_transfers(F, L, vb)) != cudaSuccess) break;
     }
   }
-  if (e == cudaSuccess) e = upload_vec(&mg.d_cls, mg.cls);
   if (e == cudaSuccess) e = upload_vec(&mg.d_blk_cls, blk_cls);
   if (e == cudaSuccess) e = upload_vec(&mg.d_blk_alpha, blk_alpha);
   if (e == cudaSuccess) e = cudaMalloc(&mg.d_status, sizeof(int));

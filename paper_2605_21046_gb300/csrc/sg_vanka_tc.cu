@@ -25,7 +25,7 @@
 //     products are exact and accumulate in FP32, so the product carries the
 //     patch values to 2^-18, 2^9 times finer than the rounding of the stored
 //     bf16 factors it multiplies.  Term t of slot s is MMA column
-//     t SLP + s (SLP = the slots rounded up to 16), so one thread writes eight
+//     t SLP + s (SLP = the slots rounded up to 8), so one thread writes eight
 //     K values of one column as a 16-byte store and consecutive slots fall in
 //     consecutive core-matrix rows.  Cell 1's K chunks follow cell 0's
 //     directly: where a K step of cell 0 reaches into them, A's columns are
