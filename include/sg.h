@@ -254,7 +254,7 @@ sg_status sg_mg_set_coarse_dofs(sg_ctx* ctx, int max_dofs);
 /* sg_mg_level_info - the choices of a built preconditioner on one level
  * (0 = finest).  info: HOST int[10] out = {number of levels, cells, 1 if the
  * coarsest (dense) level, level residual (0 the SG cell kernel with the
- * diagonal coupling table, 1 the diagonal apply, -1 none on the coarsest),
+ * diagonal coupling table, 1 the row-diagonal apply, -1 none on the coarsest),
  * Vanka cells per shared-memory chunk (tensor-core sweep: staging buffers),
  * Vanka chaos modes per tile, patch size
  * N_t (k+1)^d, diagonal classes, Vanka kernel (0 FFMA, 1 tensor cores, 2 registers),
@@ -276,9 +276,9 @@ sg_status sg_mg_setup_times(sg_ctx* ctx, double* total_ms, double* factor_ms, do
  * FFMA sweep, 1 the tensor-core sweep (SG_PREC_BF16 factors, one diagonal
  * class, patches of at most 64 unknowns, at most 80 modes per tile; the
  * transposed V-cycle keeps the FFMA sweep).
- * 2 is the register sweep (FP32 vectors, 2D patches of at most 18 unknowns;
- * it has no chunk or tile, and forcing one of those with vanka_kind -1 leaves
- * it for the FFMA sweep).
+ * A level that set-up gave the register sweep (kind 2 of sg_mg_level_info: FP32
+ * vectors, 2D patches of at most 18 unknowns; it has no chunk or tile) keeps it
+ * until a chunk, a tile or one of these sweeps is asked for.
  * The results stay the same up to rounding (the variants compute the same
  * V-cycle).  The next sg_vcycle records a new graph.  SG_ERR_ARG /
  * SG_ERR_UNSUPPORTED (nothing changed) when a level cannot take the variant.
@@ -493,8 +493,8 @@ sg_status sg_stat_errors(sg_ctx* ctx, const double* mean, const double* var, dou
  * deterministic heat equation with a(x, xi_s) = sum_mu a_mu(x) Psi_mu(xi_s) and
  * the manufactured forcing f(x, t, xi_s) of sg_set_exact is marched over all
  * slabs of the context (same mesh, Q_k and dG(r)).  All samples form one
- * block-diagonal system per slab: one Monte-Carlo apply launch covers every
- * sample (in tiles of `batch` samples), FGMRES(10) iterates on the whole
+ * block-diagonal system per slab: the apply covers every sample in waves of
+ * whole tiles of `batch` samples, FGMRES(10) iterates on the whole
  * system to rtol with a graph-captured mean-operator V-cycle as
  * preconditioner.  Samples are split into groups solved one after another
  * only when the device memory cannot hold them at once.
@@ -516,7 +516,7 @@ sg_status mc_solve_batch(sg_ctx* ctx, int n_samples, const double* xi, int batch
 /* mc_solve_meshes - mc_solve_batch for samples on several meshes at once
  * (up to 4 contexts of the same dimension, degrees, slabs, T and coefficient
  * terms; mesh sizes may differ): the samples of every mesh join ONE system
- * per slab, ONE apply launch covers every (mesh, sample tile, cell) unit, and
+ * per slab, the apply covers the samples mesh by mesh, and
  * each mesh keeps its own mean-operator V-cycle.  Per mesh p: ctxs[p],
  * n_samples[p], xi[p] (HOST n_samples[p] x M), mean_T[p], var_T[p] (DEVICE
  * n_x[p] doubles out), u_T[p] (DEVICE or NULL; u_T itself may be NULL).

@@ -13,17 +13,15 @@
 // the Gauss-point work couples every chaos mode (through G_mu) and every time
 // node (through A_t):
 //   phase 0  compute the global node of every (cell, local node) of the
-//            chunk once into shared memory, gather the chunk's nodal values
-//            of every vector through it (Dirichlet nodes read as 0), and the
-//            coefficient values of its cells, as
-//            products G value x a_mu(x_q) for each distinct (mu, G value) pair
-//            of the coupling table (13 pairs for M = 4, P = 3: the mean term's
-//            1 and sqrt(1..3) for each xi_m), so the entries below need no
-//            multiply;
-//   phase 1  per (cell, vector): sum-factorised interpolation to the
-//            (k+1)^d Gauss points and collocation gradients (reference
-//            tables are compile-time constants, so their exact zeros and ones
-//            cost nothing);
+//            chunk once into shared memory (double-word also gathers and
+//            converts the chunk's nodal values here), and stage the
+//            coefficient values of its cells, as products G value x a_mu(x_q)
+//            for each distinct (mu, G value) pair of the coupling table (13
+//            pairs for M = 4, P = 3: the mean term's 1 and sqrt(1..3) for each
+//            xi_m), so the entries below need no multiply;
+//   phase 1  per (cell, vector): gather its nodal values (Dirichlet nodes read
+//            as 0), sum-factorised interpolation to the (k+1)^d Gauss points
+//            and gradients, by the even and odd parts of every line;
 //   phase 2  per (cell, Gauss point, alpha): the time-node mass coupling
 //            w_q sum_j A_t[i][j] u[alpha,j] and the sparse chaos contraction
 //            sum_(beta,mu) G_mu[alpha][beta] a_mu(x_q) grad u[beta,i]; the
@@ -34,8 +32,8 @@
 //   phase 3  per (cell, vector): the transposed sum factorisation back to
 //            the cell's nodes;
 //   phase 4  per (cell, vector, node): scale by tau*Bhat_ii and add into y
-//            with an FP64 atomic in L2 (y was set by the init kernel: x on
-//            Dirichlet nodes, 0 elsewhere).
+//            with an FP64 atomic in L2 (y is set by the start pass: x on
+//            Dirichlet nodes, 0 elsewhere; the cell kernel waits for it here).
 // The kernel is generic over its arithmetic (sg_arith.h): native FP64, or
 // double-word FP32 pairs that run on the FP32 pipe (58x the FP64 rate on
 // GB300) with error-free transformations.  The device code is in

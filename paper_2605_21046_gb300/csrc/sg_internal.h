@@ -280,7 +280,7 @@ void mg_free(MG& mg);
 sg_status mg_level_info(const MG& mg, int level, int info[10], std::string& msg);
 // Forces the level residual kind (-1 keep, 0 cell kernel, 1 diagonal apply),
 // the Vanka cells per chunk (0 keep), modes per tile (-1 keep, 0 all) and
-// Vanka kernel (-1 keep, 0 FFMA, 1 tensor cores, 2 registers) on one smoothed level (or
+// Vanka kernel (-1 keep, 0 FFMA, 1 tensor cores) on one smoothed level (or
 // every one with level = -1); drops the captured graphs.
 sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int tile, int kind, std::string& msg);
 // The stored inverse of the Vanka patch of (mode alpha's class, cell) on a

@@ -1880,7 +1880,7 @@ sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int 
     msg = "level out of range";
     return SG_ERR_ARG;
   }
-  if (residual_kind < -1 || residual_kind > 1 || chunk < 0 || chunk > 8 || tile < -1 || kind < -1 || kind > 2) {
+  if (residual_kind < -1 || residual_kind > 1 || chunk < 0 || chunk > 8 || tile < -1 || kind < -1 || kind > 1) {
     msg = "variant out of range";
     return SG_ERR_ARG;
   }
@@ -1907,16 +1907,7 @@ sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int 
       // the register sweep has no chunk or tile: asking for one asks for the FFMA sweep
       const int kd = kind >= 0 ? kind : (L.vanka_kind == 2 && (chunk > 0 || tile >= 0) ? 0 : L.vanka_kind);
       if (kd == 2) {
-        if (!L.d_inv_col) {
-          msg = "the register Vanka sweep needs FP32 vectors and a 2D patch of at most 18 unknowns";
-          return SG_ERR_UNSUPPORTED;
-        }
-        if (pass == 1) {
-          if (residual_kind >= 0) L.use_diag = residual_kind == 1;
-          L.vanka_kind = kd;
-          L.vanka_chunk = L.ffma_chunk;
-          L.vanka_tile = L.ffma_tile;
-        }
+        if (pass == 1 && residual_kind >= 0) L.use_diag = residual_kind == 1;
         continue;
       }
       // "keep" of a sweep that is not running: the FFMA sweep's last chunk and
