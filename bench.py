@@ -64,18 +64,22 @@ def fp64_peak_tflops(sm_max_mhz=None):
     mhz = sm_max_mhz or peaks().get("sm_max_mhz") or 2070.0
     FP64_PEAK_TFLOPS = n_sm * FP64_FMA_PER_SM_CLOCK * 2 * float(mhz) * 1e6 / 1e12
     return FP64_PEAK_TFLOPS
-# algorithmic work of the sum-factorised apply per unknown (FP64 flop) and
-# the algorithmic HBM bytes per unknown (read x, write y once)
+# algorithmic work of the sum-factorised apply per unknown (FP64 flop, counted
+# for the dense 1D tables: the kernel's even/odd passes need 30 % fewer, so the
+# rate in these units can exceed the FP64 peak; FP64_INSTR_PER_UNKNOWN is what
+# it issues, 236 per cell and vector on 64x64 Q2) and the algorithmic HBM bytes
+# per unknown (read x, write y once)
 FLOP_PER_UNKNOWN = 166.0
+FP64_INSTR_PER_UNKNOWN = 236.0 * 4096 * 70 / 1_164_870
 BYTES_PER_UNKNOWN = 16.0
 L2_BYTES = 135_528_448
 # V-cycle smoothing used by the solve measurements: one pre- and one
 # post-smoothing Vanka step with damping 0.9 reaches 1e-8 fastest on GB300
-# (2D: 9 iterations, 8.3 ms vs 8 iterations, 10.2 ms with nu = 2, omega = 0.7)
+# (2D, with earlier kernels: 9 iterations, 8.3 ms vs 8 iterations, 10.2 ms with nu = 2, omega = 0.7)
 MG_NU, MG_OMEGA = 1, 0.9
 # dram__bytes_read.sum + dram__bytes_write.sum of one FP64 chunk-kernel launch on
 # this workload (ncu capture summarised in profiles/); None once the kernel changes
-NCU_TRAFFIC_BYTES = 19_920_640 + 0
+NCU_TRAFFIC_BYTES = 19_930_000 + 2_300
 
 
 def workload():
@@ -521,6 +525,7 @@ def run_ours(args, world, rank, local):
                     "synchronous": {"value": e2e_sync, "api": "sg_apply_host (returns when y is on the host)"}},
             "roofline": {"bound": "alu", "achieved": achieved_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": achieved_tf / FP64_PEAK_TFLOPS, "traffic": NCU_TRAFFIC_BYTES,
+                         "fp64_issue_frac": FP64_INSTR_PER_UNKNOWN * n / t_launch / 1e12 / (FP64_PEAK_TFLOPS / 2),
                          "kernel": "sg_apply (init + chunk kernel, per-launch CUDA events)",
                          "hbm": {"achieved": hbm_gbs, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                                  "frac": hbm_gbs / pk.get("hbm_gbs", 6800.0)}},
