@@ -223,12 +223,13 @@ struct MGLevel {
   // transfers to (down) and from (up) the next coarser level: per direction
   // the 1D lists, padded to `width` entries per output (weight 0) and stored
   // entry-major, [entry][output], weights in the MG precision; `tile` output
-  // rows per block and the input rows of every tile
+  // rows per block and the input rows of every tile; tile_x > 0: tiles of that
+  // many columns as well, and the input columns of every one
   struct Transfer {
     int* idx[3] = {nullptr, nullptr, nullptr};
     void* w[3] = {nullptr, nullptr, nullptr};
-    int* range = nullptr;
-    int width = 0, tile = 0, max_rows = 0;
+    int *range = nullptr, *range_x = nullptr;
+    int width = 0, tile = 0, max_rows = 0, tile_x = 0, max_cols = 0;
     size_t smem = 0;
   } down, up;
 };

@@ -451,6 +451,12 @@ __global__ void __launch_bounds__(256, 2) mg_vanka(const VankaParams<T> p) {
 // output's neighbours use) and stored entry-major; a thread keeps one output
 // column, with its list in registers, and walks the rows.
 //
+// LARGE: the block takes a tile of columns along x as well, with its own
+// input window, and its place comes from a 1D grid, so no length of a row and
+// no count of rows or planes is too large.  build_transfers takes it only where
+// the other form cannot be launched: whole rows need no division per value,
+// and each further tile of columns loads a halo of its own.
+//
 // The vectors that the next kernels reduce into are preset here, where their
 // nodes are written anyway: restriction also writes the coarse level's start
 // (x = 0, r = b; b vanishes on the boundary), interpolation r = b inside and 0
@@ -466,20 +472,63 @@ struct TransferParams {
   T *out, *x, *r;           // restriction: b, x, r of the coarse level; interpolation: fine x (out), r
   const int* idx[3];
   const T* w[3];
-  const int* range;         // first and number of input rows of every tile
+  const int *range, *range_x;   // first and number of input rows (columns) of every tile
   long long n_in, n_out;    // nodes per vector
   int ni[3], no[3];         // nodes per direction of the input and output grids
   int tile, max_rows, z;    // output rows per tile, most input rows of one; 3D
+  int tile_x, max_cols;     // output columns per tile, most input columns of one (LARGE)
+  unsigned n_vec, planes, tiles;   // vectors, planes and tiles of rows (LARGE)
   int cb_in, cb_out;        // columns a pass takes at a time, of the input and output grids
   long long lim_in, lim_out;   // values of the vectors (bounds checks)
 };
 
-// The input rows [lo, lo + cnt) of the tile, combined along z, into S0 (row pitch ni[0]).
-template <typename T, int W>
-__device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz, int lo, int cnt, T* S0) {
-  const long long v_in = (long long)blockIdx.x * p.n_in;
+// The part of a transfer that a block takes: vector, plane, output rows
+// [j0, j0 + nj) and columns [i0, i0 + ni), input rows [lo, lo + cnt) and
+// columns [lox, lox + cntx).
+struct TransferTile {
+  int v, jz, j0, nj, i0, ni, lo, cnt, lox, cntx;
+};
+template <typename T, bool LARGE>
+__device__ __forceinline__ TransferTile transfer_tile(const TransferParams<T>& p) {
+  TransferTile t;
+  unsigned ty = blockIdx.z;
+  if constexpr (LARGE) {
+    unsigned b = blockIdx.x;
+    t.v = (int)(b % p.n_vec);
+    b /= p.n_vec;
+    t.jz = (int)(b % p.planes);
+    b /= p.planes;
+    ty = b % p.tiles;
+    b /= p.tiles;
+    t.i0 = (int)b * p.tile_x;
+    t.ni = min(p.tile_x, p.no[0] - t.i0);
+    t.lox = __ldg(p.range_x + 2 * b);
+    t.cntx = __ldg(p.range_x + 2 * b + 1);
+  } else {
+    t.v = (int)blockIdx.x;
+    t.jz = (int)blockIdx.y;
+    t.i0 = t.lox = 0;
+    t.ni = p.no[0];
+    t.cntx = p.ni[0];
+  }
+  t.j0 = (int)ty * p.tile;
+  t.nj = min(p.tile, p.no[1] - t.j0);
+  t.lo = __ldg(p.range + 2 * ty);
+  t.cnt = __ldg(p.range + 2 * ty + 1);
+  return t;
+}
+
+// The tile's input rows, combined along z, into S0 (row pitch cntx).
+template <typename T, int W, bool LARGE>
+__device__ __forceinline__ void transfer_load(const TransferParams<T>& p, const TransferTile& t, T* S0) {
+  const int jz = t.jz;
+  const long long v_in = (long long)t.v * p.n_in;
   const T* src = p.in + v_in;
-  const int n = cnt * p.ni[0], off = lo * p.ni[0];
+  const int n = t.cnt * t.cntx, off = t.lo * p.ni[0] + t.lox;
+  auto at = [&](int i) {   // of the tile's value i, from its first one
+    if constexpr (LARGE) return (i / t.cntx) * p.ni[0] + i % t.cntx;
+    else return i;
+  };
   if (p.z) {
     const int plane = p.ni[0] * p.ni[1];
     const T* pl[W];
@@ -502,7 +551,7 @@ __device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz
 #pragma unroll
         for (int g = 0; g < kTransferBatch; ++g) {
           const int i = i0 + g * kTransferThreads;
-          if (i < n && SG_IN(pl[k] - p.in + i, p.lim_in, 501)) s[g] = fma(wz[k], __ldg(pl[k] + i), s[g]);
+          if (i < n && SG_IN(pl[k] - p.in + at(i), p.lim_in, 501)) s[g] = fma(wz[k], __ldg(pl[k] + at(i)), s[g]);
         }
       }
 #pragma unroll
@@ -515,7 +564,7 @@ __device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz
 #pragma unroll
       for (int g = 0; g < kTransferBatch; ++g) {
         const int i = i0 + g * kTransferThreads;
-        s[g] = i < n && SG_IN(v_in + off + i, p.lim_in, 501) ? __ldg(src + off + i) : T(0);
+        s[g] = i < n && SG_IN(v_in + off + at(i), p.lim_in, 501) ? __ldg(src + off + at(i)) : T(0);
       }
 #pragma unroll
       for (int g = 0; g < kTransferBatch; ++g)
@@ -524,11 +573,11 @@ __device__ __forceinline__ void transfer_load(const TransferParams<T>& p, int jz
   }
 }
 
-// One 1D pass along x or y of `rows` output rows: DIR 0 out[row][c] = sum_k w in[row][idx[c]],
-// DIR 1 out[row][c] = sum_k w in[idx[row0 + row] - lo][c]; put(row, column, value).
+// One 1D pass along x or y of `rows` output rows: DIR 0 out[row][c] = sum_k w in[row][idx[o0 + c] - lo],
+// DIR 1 out[row][c] = sum_k w in[idx[o0 + row] - lo][c]; put(row, column, value).
 template <typename T, int W, int DIR, class Put>
 __device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, int cb, int rows, const int* idx,
-                                              const T* w, int n_list, int row0, int lo, Put put) {
+                                              const T* w, int n_list, int o0, int lo, Put put) {
   const int par = kTransferThreads / cb;                       // cb columns x par rows at a time
   const int c0 = threadIdx.x % cb, r0 = threadIdx.x / cb;
   if (r0 >= par) return;
@@ -538,8 +587,8 @@ __device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, 
       T wt[W];
 #pragma unroll
       for (int k = 0; k < W; ++k) {
-        at[k] = __ldg(idx + k * n_list + c);
-        wt[k] = __ldg(w + k * n_list + c);
+        at[k] = __ldg(idx + k * n_list + o0 + c) - lo;
+        wt[k] = __ldg(w + k * n_list + o0 + c);
       }
       for (int r = r0; r < rows; r += par) {
         T s = T(0);
@@ -552,28 +601,27 @@ __device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, 
         T s = T(0);
 #pragma unroll
         for (int k = 0; k < W; ++k)
-          s = fma(__ldg(w + k * n_list + row0 + r), in[(__ldg(idx + k * n_list + row0 + r) - lo) * pitch + c], s);
+          s = fma(__ldg(w + k * n_list + o0 + r), in[(__ldg(idx + k * n_list + o0 + r) - lo) * pitch + c], s);
         put(r, c, s);
       }
     }
   }
 }
 
-template <typename T, int W>
+template <typename T, int W, bool LARGE>
 __global__ void __launch_bounds__(kTransferThreads) mg_restrict(const TransferParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][fine x]
-  T* S1 = S0 + (size_t)p.max_rows * p.ni[0];                    // [max_rows][coarse x]
-  const int jz = blockIdx.y, j0 = blockIdx.z * p.tile, nj = min(p.tile, p.no[1] - j0);
-  const int lo = __ldg(p.range + 2 * blockIdx.z), cnt = __ldg(p.range + 2 * blockIdx.z + 1);
-  transfer_load<T, W>(p, jz, lo, cnt, S0);
+  const TransferTile t = transfer_tile<T, LARGE>(p);
+  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][fine columns]
+  T* S1 = S0 + (size_t)p.max_rows * (LARGE ? p.max_cols : p.ni[0]);   // [max_rows][coarse columns]
+  transfer_load<T, W, LARGE>(p, t, S0);
   __syncthreads();
-  const int ncx = p.no[0];
-  transfer_pass<T, W, 0>(S0, p.ni[0], ncx, p.cb_out, cnt, p.idx[0], p.w[0], ncx, 0, 0,
-                         [&](int r, int c, T v) { S1[r * ncx + c] = v; });
+  const int ncx = p.no[0], nc = LARGE ? t.ni : ncx;
+  transfer_pass<T, W, 0>(S0, t.cntx, nc, p.cb_out, t.cnt, p.idx[0], p.w[0], ncx, t.i0, t.lox,
+                         [&](int r, int c, T v) { S1[r * nc + c] = v; });
   __syncthreads();
-  const long long o0 = (long long)blockIdx.x * p.n_out + ((long long)jz * p.no[1] + j0) * ncx;
-  transfer_pass<T, W, 1>(S1, ncx, ncx, p.cb_out, nj, p.idx[1], p.w[1], p.no[1], j0, lo, [&](int r, int c, T v) {
+  const long long o0 = (long long)t.v * p.n_out + ((long long)t.jz * p.no[1] + t.j0) * ncx + t.i0;
+  transfer_pass<T, W, 1>(S1, nc, nc, p.cb_out, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo, [&](int r, int c, T v) {
     const long long o = o0 + (long long)r * ncx + c;
     if (!SG_IN(o, p.lim_out, 502)) return;
     p.out[o] = v;
@@ -582,44 +630,48 @@ __global__ void __launch_bounds__(kTransferThreads) mg_restrict(const TransferPa
   });
 }
 
-template <typename T, int W>
+template <typename T, int W, bool LARGE>
 __global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][coarse x]
-  T* S1 = S0 + (size_t)p.max_rows * p.ni[0];                    // [tile][coarse x]
-  T* S2 = S1 + (size_t)p.tile * p.ni[0];                        // [tile][fine x]
-  const int jz = blockIdx.y, j0 = blockIdx.z * p.tile, nj = min(p.tile, p.no[1] - j0);
-  const int lo = __ldg(p.range + 2 * blockIdx.z), cnt = __ldg(p.range + 2 * blockIdx.z + 1);
-  transfer_load<T, W>(p, jz, lo, cnt, S0);
+  const TransferTile t = transfer_tile<T, LARGE>(p);
+  const int most = LARGE ? p.max_cols : p.ni[0];
+  T* S0 = reinterpret_cast<T*>(smem_raw);                       // [max_rows][coarse columns]
+  T* S1 = S0 + (size_t)p.max_rows * most;                       // [tile][coarse columns]
+  T* S2 = S1 + (size_t)p.tile * most;                           // [tile][fine columns]
+  transfer_load<T, W, LARGE>(p, t, S0);
   __syncthreads();
-  const int ncx = p.ni[0], nfx = p.no[0];
-  transfer_pass<T, W, 1>(S0, ncx, ncx, p.cb_in, nj, p.idx[1], p.w[1], p.no[1], j0, lo,
-                         [&](int r, int c, T v) { S1[r * ncx + c] = v; });
+  const int nfx = p.no[0];
+  transfer_pass<T, W, 1>(S0, t.cntx, t.cntx, p.cb_in, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo,
+                         [&](int r, int c, T v) { S1[r * t.cntx + c] = v; });
   __syncthreads();
-  transfer_pass<T, W, 0>(S1, ncx, nfx, p.cb_out, nj, p.idx[0], p.w[0], nfx, 0, 0,
-                         [&](int r, int c, T v) { S2[r * nfx + c] = v; });
+  transfer_pass<T, W, 0>(S1, t.cntx, t.ni, p.cb_out, t.nj, p.idx[0], p.w[0], nfx, t.i0, t.lox,
+                         [&](int r, int c, T v) { S2[r * t.ni + c] = v; });
   __syncthreads();
-  // the tile's rows are contiguous: x += S2, r = b inside, with the loads of a batch in flight together
-  const long long o0 = (long long)blockIdx.x * p.n_out + ((long long)jz * p.no[1] + j0) * nfx;
-  const bool edge_z = p.z && (jz == 0 || jz == p.no[2] - 1);
-  const int n = nj * nfx;
+  // x += S2, r = b inside (whole rows of a tile are contiguous), with the loads of a batch in flight together
+  const long long o0 = (long long)t.v * p.n_out + ((long long)t.jz * p.no[1] + t.j0) * nfx + t.i0;
+  const bool edge_z = p.z && (t.jz == 0 || t.jz == p.no[2] - 1);
+  const int n = t.nj * t.ni;
+  auto at = [&](int i) {
+    if constexpr (LARGE) return o0 + (long long)(i / t.ni) * nfx + i % t.ni;
+    else return o0 + i;
+  };
   for (int i0 = threadIdx.x; i0 < n; i0 += kTransferBatch * kTransferThreads) {
     T xv[kTransferBatch], bv[kTransferBatch];
 #pragma unroll
     for (int g = 0; g < kTransferBatch; ++g) {
       const int i = i0 + g * kTransferThreads;
-      const bool in = i < n && SG_IN(o0 + i, p.lim_out, 503);
-      xv[g] = in ? p.out[o0 + i] : T(0);
-      bv[g] = in ? __ldg(p.b + o0 + i) : T(0);
+      const bool in = i < n && SG_IN(at(i), p.lim_out, 503);
+      xv[g] = in ? p.out[at(i)] : T(0);
+      bv[g] = in ? __ldg(p.b + at(i)) : T(0);
     }
 #pragma unroll
     for (int g = 0; g < kTransferBatch; ++g) {
       const int i = i0 + g * kTransferThreads;
-      if (i >= n || !SG_IN(o0 + i, p.lim_out, 503)) continue;
-      const int r = i / nfx, c = i - r * nfx, jy = j0 + r;
+      if (i >= n || !SG_IN(at(i), p.lim_out, 503)) continue;
+      const int r = i / t.ni, c = t.i0 + i - r * t.ni, jy = t.j0 + r;
       const bool bd = edge_z || jy == 0 || jy == p.no[1] - 1 || c == 0 || c == nfx - 1;
-      p.out[o0 + i] = xv[g] + S2[i];
-      p.r[o0 + i] = bd ? T(0) : bv[g];
+      p.out[at(i)] = xv[g] + S2[i];
+      p.r[at(i)] = bd ? T(0) : bv[g];
     }
   }
 }
@@ -1213,13 +1265,19 @@ void transfer_params(const MGLevel& I, const MGLevel& O, const MGLevel::Transfer
     p.no[d] = O.hp.nn[d];
   }
   p.range = t.range;
+  p.range_x = t.range_x;
   p.n_in = I.hp.n_x;
   p.n_out = O.hp.n_x;
   p.tile = t.tile;
   p.max_rows = t.max_rows;
   p.z = I.hp.dim == 3;
-  p.cb_in = column_block(p.ni[0]);
-  p.cb_out = column_block(p.no[0]);
+  p.tile_x = t.tile_x;
+  p.max_cols = t.max_cols;
+  p.n_vec = (unsigned)V;
+  p.planes = (unsigned)p.no[2];
+  p.tiles = (unsigned)((p.no[1] + t.tile - 1) / t.tile);
+  p.cb_in = column_block(t.tile_x > 0 ? t.max_cols : p.ni[0]);
+  p.cb_out = column_block(t.tile_x > 0 ? t.tile_x : p.no[0]);
   p.lim_in = (long long)V * I.hp.n_x;
   p.lim_out = (long long)V * O.hp.n_x;
 }
@@ -1229,6 +1287,14 @@ void transfer_params(const MGLevel& I, const MGLevel& O, const MGLevel::Transfer
 // with coarse and then fine rows).
 size_t transfer_smem(bool up, int max_rows, int tile, int nfx, int ncx, size_t vb) {
   return vb * (up ? (size_t)max_rows * ncx + (size_t)tile * (ncx + nfx) : (size_t)max_rows * (nfx + ncx));
+}
+
+// The launch grid of a transfer: vectors, planes and tiles of rows, or all of
+// them and the tiles of columns on x.
+template <typename T>
+dim3 transfer_grid(const TransferParams<T>& p, const MGLevel::Transfer& t) {
+  if (t.tile_x == 0) return dim3(p.n_vec, p.planes, p.tiles);
+  return dim3((unsigned)((size_t)p.n_vec * p.planes * p.tiles * ((p.no[0] + t.tile_x - 1) / t.tile_x)));
 }
 
 #define SG_TRANSFER_WIDTHS(CALL) \
@@ -1252,8 +1318,10 @@ cudaError_t prolong(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
   p.out = static_cast<T*>(F.d_x);
   p.x = nullptr;
   p.r = static_cast<T*>(F.d_r);
-  const dim3 grid(V, p.z ? p.no[2] : 1, (p.no[1] + t.tile - 1) / t.tile);
-#define SG_CALL(W) mg_prolong<T, W><<<grid, kTransferThreads, t.smem, s>>>(p)
+  const dim3 grid = transfer_grid(p, t);
+#define SG_CALL(W)                                                                  \
+  if (t.tile_x > 0) mg_prolong<T, W, true><<<grid, kTransferThreads, t.smem, s>>>(p); \
+  else mg_prolong<T, W, false><<<grid, kTransferThreads, t.smem, s>>>(p)
   SG_TRANSFER_WIDTHS(SG_CALL)
 #undef SG_CALL
   return cudaGetLastError();
@@ -1270,8 +1338,10 @@ cudaError_t restrict_to(MGLevel& F, MGLevel& C, int V, cudaStream_t s) {
   p.out = static_cast<T*>(C.d_b);
   p.x = static_cast<T*>(C.d_x);
   p.r = static_cast<T*>(C.d_r);
-  const dim3 grid(V, p.z ? p.no[2] : 1, (p.no[1] + t.tile - 1) / t.tile);
-#define SG_CALL(W) mg_restrict<T, W><<<grid, kTransferThreads, t.smem, s>>>(p)
+  const dim3 grid = transfer_grid(p, t);
+#define SG_CALL(W)                                                                  \
+  if (t.tile_x > 0) mg_restrict<T, W, true><<<grid, kTransferThreads, t.smem, s>>>(p); \
+  else mg_restrict<T, W, false><<<grid, kTransferThreads, t.smem, s>>>(p)
   SG_TRANSFER_WIDTHS(SG_CALL)
 #undef SG_CALL
   return cudaGetLastError();
@@ -1518,6 +1588,7 @@ void mg_free(MG& mg) {
         cudaFree(t->w[d]);
       }
       cudaFree(t->range);
+      cudaFree(t->range_x);
     }
   }
   mg.lv.clear();
@@ -1535,8 +1606,8 @@ static cudaError_t prepare_coarse(int precision) {
 // more than about 1000 nodes).
 template <typename T, int W>
 static cudaError_t prepare_transfers_w(int optin) {
-  cudaError_t e = cudaFuncSetAttribute(&mg_restrict<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-  return e == cudaSuccess ? cudaFuncSetAttribute(&mg_prolong<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)
+  cudaError_t e = cudaFuncSetAttribute(&mg_restrict<T, W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  return e == cudaSuccess ? cudaFuncSetAttribute(&mg_prolong<T, W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)
                           : e;
 }
 template <typename T>
@@ -1559,6 +1630,9 @@ static cudaError_t prepare_transfers(size_t vb) {
 // Rows per tile: halved from the whole plane until a block's rows fit in 48 KB
 // of shared memory and the blocks cover the GPU four times, or 4 rows are left
 // (64^2 Q2, 70 vectors: 8 rows, 630 blocks; 32^3 Q2: whole planes of 65 rows).
+// Where a row does not fit at all (FP64 from 6456 cells of Q1 along x, 1384 of
+// Q2 and 588 of Q3; twice that in FP32), or the grid has more than 65535 planes
+// or tiles: tiles of 8 rows, and columns halved until a block takes 48 KB.
 static cudaError_t build_transfers(MGLevel& F, const MGLevel& C, size_t vb) {
   std::vector<int> ptr[2][3], idx[2][3];
   std::vector<double> w[2][3];
@@ -1569,15 +1643,19 @@ static cudaError_t build_transfers(MGLevel& F, const MGLevel& C, size_t vb) {
       for (size_t i = 0; i + 1 < ptr[u][d].size(); ++i) longest[u] = std::max(longest[u], ptr[u][d][i + 1] - ptr[u][d][i]);
   }
   cudaError_t e = cudaSuccess;
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int precision = vb == 4 ? kPrecF32 : SG_PREC_FP64;
   for (int u = 0; u < 2; ++u) {
     MGLevel::Transfer& t = u ? F.up : F.down;
     if (longest[u] > kAxisMax) return cudaErrorInvalidValue;
     t.width = axis_width(longest[u]);
-    std::vector<int> pi, py;
+    std::vector<int> pi, px, py;
     std::vector<double> pw;
     for (int d = 0; d < F.hp.dim; ++d) {
       pad_lists(ptr[u][d], idx[u][d], w[u][d], t.width, pi, pw);
+      if (d == 0) px = pi;
       if (d == 1) py = pi;
       if ((e = upload_vec(&t.idx[d], pi)) != cudaSuccess) return e;
       if ((e = upload_values(&t.w[d], pw, precision)) != cudaSuccess) return e;
@@ -1592,6 +1670,19 @@ static cudaError_t build_transfers(MGLevel& F, const MGLevel& C, size_t vb) {
       const long long blocks = planes * ((out.nn[1] + t.tile - 1) / t.tile);
       if (t.tile == 1 || (t.smem <= 48 * 1024 && (blocks >= 4 * sg::sm_count() || t.tile <= 4))) break;
       t.tile = (t.tile + 1) / 2;
+    }
+    if (t.smem > (size_t)optin || out.nn[2] > 65535 || (out.nn[1] + t.tile - 1) / t.tile > 65535) {
+      std::vector<int> rx;
+      t.tile = std::min(8, out.nn[1]);
+      t.tile_x = out.nn[0];
+      t.max_rows = tile_ranges(py, t.width, out.nn[1], t.tile, range);
+      while (true) {
+        t.max_cols = tile_ranges(px, t.width, out.nn[0], t.tile_x, rx);
+        t.smem = transfer_smem(u == 1, t.max_rows, t.tile, u ? t.tile_x : t.max_cols, u ? t.max_cols : t.tile_x, vb);
+        if (t.smem <= 48 * 1024 || t.tile_x == 1) break;
+        t.tile_x = (t.tile_x + 1) / 2;
+      }
+      if ((e = upload_vec(&t.range_x, rx)) != cudaSuccess) return e;
     }
     if (t.smem > 48 * 1024 && (e = prepare_transfers(vb)) != cudaSuccess) return e;
     if ((e = upload_vec(&t.range, range)) != cudaSuccess) return e;
