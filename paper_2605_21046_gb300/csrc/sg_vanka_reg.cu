@@ -119,22 +119,26 @@ __global__ void __launch_bounds__(32 * kRegWarps) mg_vanka_reg(const RegVankaArg
     }
 }
 
-// inv [class][cell][np][npp] (float or bf16) -> out [class][np * np][cell], 32 x 32 tiles through shared memory
+// inv [class][cell][np][npp] (float or bf16) -> out [class][np * np][cell], 32 x 32 tiles through shared
+// memory; cells on grid.x, which alone takes more than 65535 tiles of them
 template <typename W>
 __global__ void __launch_bounds__(256) vanka_columns(const W* __restrict__ in, float* __restrict__ out, int np, int npp,
-                                                     int n_cells) {
+                                                     int n_cells, int n_classes) {
   __shared__ float tile[32][33];
-  const int cls = blockIdx.z, e0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  const W* src = in + (long long)cls * n_cells * np * npp;
-  float* dst = out + (long long)cls * np * np * n_cells;
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int c = c0 + j, e = e0 + threadIdx.x;
-    if (c < n_cells && e < np * np) tile[j][threadIdx.x] = (float)src[((long long)c * np + e / np) * npp + e % np];
-  }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int e = e0 + j, c = c0 + threadIdx.x;
-    if (c < n_cells && e < np * np) dst[(long long)e * n_cells + c] = tile[threadIdx.x][j];
+  const int c0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
+  for (int cls = blockIdx.z; cls < n_classes; cls += gridDim.z) {
+    const W* src = in + (long long)cls * n_cells * np * npp;
+    float* dst = out + (long long)cls * np * np * n_cells;
+    for (int j = threadIdx.y; j < 32; j += 8) {
+      const int c = c0 + j, e = e0 + threadIdx.x;
+      if (c < n_cells && e < np * np) tile[j][threadIdx.x] = (float)src[((long long)c * np + e / np) * npp + e % np];
+    }
+    __syncthreads();
+    for (int j = threadIdx.y; j < 32; j += 8) {
+      const int e = e0 + j, c = c0 + threadIdx.x;
+      if (c < n_cells && e < np * np) dst[(long long)e * n_cells + c] = tile[threadIdx.x][j];
+    }
+    __syncthreads();
   }
 }
 
@@ -148,9 +152,9 @@ cudaError_t vanka_reg_columns(const void* inv, bool bf16, int np, int npp, int n
   const size_t n = (size_t)n_classes * np * np * n_cells;
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(out), n * sizeof(float));
   if (e != cudaSuccess) return e;
-  const dim3 grid((np * np + 31) / 32, (unsigned)((n_cells + 31) / 32), n_classes), block(32, 8);
-  if (bf16) vanka_columns<<<grid, block>>>(static_cast<const __nv_bfloat16*>(inv), *out, np, npp, (int)n_cells);
-  else vanka_columns<<<grid, block>>>(static_cast<const float*>(inv), *out, np, npp, (int)n_cells);
+  const dim3 grid((unsigned)((n_cells + 31) / 32), (np * np + 31) / 32, std::min(n_classes, 65535)), block(32, 8);
+  if (bf16) vanka_columns<<<grid, block>>>(static_cast<const __nv_bfloat16*>(inv), *out, np, npp, (int)n_cells, n_classes);
+  else vanka_columns<<<grid, block>>>(static_cast<const float*>(inv), *out, np, npp, (int)n_cells, n_classes);
   return cudaGetLastError();
 }
 
