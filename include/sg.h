@@ -279,6 +279,8 @@ sg_status sg_mg_setup_times(sg_ctx* ctx, double* total_ms, double* factor_ms, do
  * A level that set-up gave the register sweep (kind 2 of sg_mg_level_info: FP32
  * vectors, 2D patches of at most 18 unknowns; it has no chunk or tile) keeps it
  * until a chunk, a tile or one of these sweeps is asked for.
+ * Its inverses are then put back in the order of the other sweeps (SG_ERR_OOM,
+ * nothing changed, without room for both orders of a level at once).
  * The results stay the same up to rounding (the variants compute the same
  * V-cycle).  The next sg_vcycle records a new graph.  SG_ERR_ARG /
  * SG_ERR_UNSUPPORTED (nothing changed) when a level cannot take the variant.

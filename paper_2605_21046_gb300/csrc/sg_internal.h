@@ -210,7 +210,8 @@ struct MGLevel {
   bool chunk_ok = false;     // the SG cell kernel has a launch shape for this level
   void* d_inv = nullptr;     // [class][cell][np][pitch] patch inverses (pitch = np rounded up to 8;
                              //  bf16 when MG::bf16), or coarsest [class][n_int][n_int]
-  float* d_inv_col = nullptr;   // [class][entry][cell]: the inverses of the register sweep (null: it does not apply)
+  void* d_inv_col = nullptr; // [class][np * np][cell]: the same in the register sweep's order, in place of d_inv
+                             //  (a level holds one of the two: this one while vanka_kind is 2)
   int vanka_chunk = 0;       // cells per Vanka chunk
   int vanka_tile = 0;        // modes per Vanka tile on this level (0: the multigrid's tile)
   int vanka_kind = 0;        // Vanka sweep: 0 FFMA kernel, 1 tensor-core kernel (bf16 factors), 2 register kernel
@@ -303,12 +304,14 @@ cudaError_t launch_vanka_tc(const HostProblem& hp, const float* r, float* x, con
 // ok = false where that fails or its check does; out is then undefined.
 cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int precision, void* out, bool& ok);
 // The register Vanka sweep (2D patches of at most 18 unknowns, FP32 vectors;
-// sg_vanka_reg.cu): whether a shape can take it, its copy of the inverses
-// (allocates *out), and one sweep.
+// sg_vanka_reg.cu): whether a shape can take it, the inverses in its order or
+// back in the order by cell (allocates *out; synchronous), and one sweep.
 bool vanka_reg_eligible(int dim, int k, int nt);
-cudaError_t vanka_reg_columns(const void* inv, bool bf16, int np, int npp, int n_classes, long long n_cells, float** out);
-cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, const float* inv, const int* blk_cls,
-                             const int* blk_alpha, int n_blk, int n_classes, float omega, int trans, cudaStream_t s);
+cudaError_t vanka_reg_reorder(bool to_columns, const void* in, bool bf16, int np, int npp, int n_classes,
+                              long long n_cells, void** out);
+cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, const void* inv, bool bf16,
+                             const int* blk_cls, const int* blk_alpha, int n_blk, int n_classes, float omega, int trans,
+                             cudaStream_t s);
 // Vanka patch inverses of one multigrid level, assembled and inverted in FP64
 // on the device (Gauss-Jordan, partial pivoting) for every class and cell:
 // out[class][cell][np][npp] as double (out_kind 0), float (1) or bf16 (2).

@@ -1158,8 +1158,8 @@ cudaError_t launch_vanka(MG& mg, MGLevel& L, cudaStream_t s, int trans) {
   if constexpr (std::is_same<T, float>::value) {
     if (L.vanka_kind == 2)
       return launch_vanka_reg(L.hp, static_cast<const float*>(L.vanka_r ? L.vanka_r : L.d_r), static_cast<float*>(L.d_x),
-                              L.d_inv_col, mg.d_blk_cls, mg.d_blk_alpha, mg.n_blk, mg.n_classes, (float)mg.omega, trans,
-                              s);
+                              L.d_inv_col, mg.bf16, mg.d_blk_cls, mg.d_blk_alpha, mg.n_blk, mg.n_classes,
+                              (float)mg.omega, trans, s);
     if (mg.bf16 && L.vanka_kind == 1 && !trans) {
       const int tile = L.vanka_tile > 0 ? L.vanka_tile : mg.vanka_tile;
       const float* r = static_cast<const float*>(L.vanka_r ? L.vanka_r : L.d_r);
@@ -1894,9 +1894,18 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       // FP32 vectors and small 2D patches: the register sweep, always the fastest there
       // (V-cycle with it and with the tuned FFMA or tensor-core sweep: 64^2 Q2, 35 rows 0.115 and 0.158 ms; 128^2 Q2, 70 rows 0.46 and 0.70)
       if (precision == kPrecF32 && vanka_reg_eligible(L.hp.dim, L.hp.k, L.hp.n_t)) {
-        if ((e = vanka_reg_columns(L.d_inv, mg.bf16, L.np, npp, mg.n_classes, L.hp.n_cells, &L.d_inv_col)) != cudaSuccess)
-          break;
-        L.vanka_kind = 2;
+        // its order takes the place of the order by cell; without room for both at once the
+        // level keeps that one, and its sweep is timed like the others
+        e = vanka_reg_reorder(true, L.d_inv, mg.bf16, L.np, npp, mg.n_classes, L.hp.n_cells, &L.d_inv_col);
+        if (e == cudaSuccess) {
+          cudaFree(L.d_inv);
+          L.d_inv = nullptr;
+          L.vanka_kind = 2;
+        } else if (e == cudaErrorMemoryAllocation) {
+          cudaGetLastError();
+          e = cudaSuccess;
+        }
+        if (e != cudaSuccess) break;
       }
     }
     if ((e = upload_vec(&L.d_grow, L.hp.g.row)) != cudaSuccess) break;
@@ -1981,6 +1990,32 @@ sg_status mg_force_variant(MG& mg, int level, int residual_kind, int chunk, int 
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   // check every level first, then change them
   for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) {
+      // levels that leave the register sweep need their inverses by cell
+      std::vector<std::pair<MGLevel*, void*>> rows;
+      cudaError_t e = cudaSuccess;
+      for (int l = 0; l < (int)mg.lv.size() && e == cudaSuccess; ++l) {
+        MGLevel& L = mg.lv[l];
+        if ((level >= 0 && l != level) || L.coarsest || L.vanka_kind != 2 || (kind < 0 && chunk == 0 && tile < 0)) continue;
+        rows.emplace_back(&L, nullptr);
+        e = vanka_reg_reorder(false, L.d_inv_col, mg.bf16, L.np, vanka_row_pitch(L.np), mg.n_classes, L.hp.n_cells,
+                              &rows.back().second);
+      }
+      for (auto& [L, d] : rows) {
+        if (e != cudaSuccess) {
+          cudaFree(d);
+          continue;
+        }
+        L->d_inv = d;
+        cudaFree(L->d_inv_col);
+        L->d_inv_col = nullptr;
+      }
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        msg = std::string("inverses by cell: ") + cudaGetErrorString(e);
+        return e == cudaErrorMemoryAllocation ? SG_ERR_OOM : SG_ERR_CUDA;
+      }
+    }
     for (int l = 0; l < (int)mg.lv.size(); ++l) {
       if (level >= 0 && l != level) continue;
       MGLevel& L = mg.lv[l];
@@ -2060,29 +2095,32 @@ sg_status mg_patch_inverse(const MG& mg, int level, int alpha, long long cell, d
     return SG_ERR_ARG;
   }
   const int np = L.np, npp = vanka_row_pitch(np);
-  const size_t off = ((size_t)mg.cls[alpha] * L.hp.n_cells + (size_t)cell) * np * npp;
-  const size_t cnt = (size_t)np * npp;
-  std::vector<double> row(cnt);
+  const size_t wb = inv_value_bytes(mg);
+  // the patch's entries: contiguous rows, or one value of every column
+  const bool by_cell = L.d_inv != nullptr;
+  const int pitch = by_cell ? npp : np;
+  const size_t cnt = (size_t)np * pitch;
+  std::vector<unsigned char> raw(cnt * wb);
   cudaError_t e;
-  if (mg.bf16) {
-    std::vector<__nv_bfloat16> v(cnt);
-    e = cudaMemcpy(v.data(), static_cast<const __nv_bfloat16*>(L.d_inv) + off, cnt * sizeof(__nv_bfloat16),
-                   cudaMemcpyDeviceToHost);
-    for (size_t i = 0; i < cnt; ++i) row[i] = (double)__bfloat162float(v[i]);
-  } else if (mg.precision == kPrecF32) {
-    std::vector<float> v(cnt);
-    e = cudaMemcpy(v.data(), static_cast<const float*>(L.d_inv) + off, cnt * sizeof(float), cudaMemcpyDeviceToHost);
-    for (size_t i = 0; i < cnt; ++i) row[i] = v[i];
+  if (by_cell) {
+    const size_t off = ((size_t)mg.cls[alpha] * L.hp.n_cells + (size_t)cell) * cnt;
+    e = cudaMemcpy(raw.data(), static_cast<const char*>(L.d_inv) + off * wb, cnt * wb, cudaMemcpyDeviceToHost);
   } else {
-    e = cudaMemcpy(row.data(), static_cast<const double*>(L.d_inv) + off, cnt * sizeof(double),
-                   cudaMemcpyDeviceToHost);
+    const size_t off = (size_t)mg.cls[alpha] * cnt * L.hp.n_cells + (size_t)cell;
+    e = cudaMemcpy2D(raw.data(), wb, static_cast<const char*>(L.d_inv_col) + off * wb, L.hp.n_cells * wb, wb, cnt,
+                     cudaMemcpyDeviceToHost);
   }
   if (e != cudaSuccess) {
     msg = cudaGetErrorString(e);
     return SG_ERR_CUDA;
   }
   for (int r = 0; r < np; ++r)
-    for (int c = 0; c < np; ++c) out[(size_t)r * np + c] = row[(size_t)r * npp + c];
+    for (int c = 0; c < np; ++c) {
+      const unsigned char* v = raw.data() + ((size_t)r * pitch + c) * wb;
+      out[(size_t)r * np + c] = mg.bf16 ? (double)__bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(v))
+                                : mg.precision == kPrecF32 ? (double)*reinterpret_cast<const float*>(v)
+                                                           : *reinterpret_cast<const double*>(v);
+    }
   return SG_OK;
 }
 

@@ -4,7 +4,8 @@
 //
 // One thread holds one cell for one block of kVankaVB rows of a class, with the
 // patch's r values in registers; the lanes of a warp are 32 consecutive cells
-// (x fastest).  The inverses are stored [entry][cell], so a lane's entry is one
+// (x fastest).  The inverses are stored [entry][cell] in the factors' precision
+// (FP32 or bf16), so a lane's entry is one
 // coalesced load that serves kVankaVB FMAs, and a patch row's result is
 // weighted and added into x as soon as it is summed - no shared memory and no
 // barrier.  As in the row-diagonal apply the plane of nodes that a cell shares
@@ -37,7 +38,7 @@ constexpr int kRegWarps = 4;     // row blocks (warps) per thread block
 struct RegVankaArgs {
   const float* r;
   float* x;
-  const float* inv;              // [class][NP * NP][n_cells]
+  const void* inv;               // [class][NP * NP][n_cells], float or bf16
   const int* blk_cls;            // [n_blk]
   const int* blk_alpha;          // [n_blk][VB] rows, -1 padded
   long long n_x, n_vec_x, inv_count;
@@ -46,7 +47,7 @@ struct RegVankaArgs {
   float omega;
 };
 
-template <int K, int NT, bool TRANS>
+template <int K, int NT, bool TRANS, typename W>
 __global__ void __launch_bounds__(32 * kRegWarps) mg_vanka_reg(const RegVankaArgs p) {
   constexpr int N = K + 1, NKD = N * N, NP = NT * NKD;
   const int blk = blockIdx.y * kRegWarps + threadIdx.y;
@@ -79,7 +80,8 @@ __global__ void __launch_bounds__(32 * kRegWarps) mg_vanka_reg(const RegVankaArg
       }
   const bool take = valid && lane > 0 && cx > 0;                          // the left lane's last plane
   const bool give = valid && lane < 31 && cell + 1 < p.n_cells && !hi0;   // mine goes to the right lane
-  const float* inv = p.inv + (long long)__ldg(p.blk_cls + blk) * NP * NP * p.n_cells + cc;
+  const W* all = static_cast<const W*>(p.inv);
+  const W* inv = all + (long long)__ldg(p.blk_cls + blk) * NP * NP * p.n_cells + cc;
   // a line of nodes (time node i, row ay) at a time: the right lane's first
   // node needs the left lane's last one
 #pragma unroll 1
@@ -89,12 +91,12 @@ __global__ void __launch_bounds__(32 * kRegWarps) mg_vanka_reg(const RegVankaArg
 #pragma unroll
       for (int ax = 0; ax < N; ++ax) {
         const int rho = i * NKD + ay * N + ax;
-        const float* row = inv + (long long)(TRANS ? rho : rho * NP) * p.n_cells;
+        const W* row = inv + (long long)(TRANS ? rho : rho * NP) * p.n_cells;
         const long long step = (long long)(TRANS ? NP : 1) * p.n_cells;
         float w[NP];
 #pragma unroll
         for (int q = 0; q < NP; ++q)
-          w[q] = SG_IN((long long)(row - p.inv) + q * step, p.inv_count, 802) ? __ldg(row + q * step) : 0.0f;
+          w[q] = SG_IN((long long)(row - all) + q * step, p.inv_count, 802) ? (float)__ldg(row + q * step) : 0.0f;
 #pragma unroll
         for (int u = 0; u < VB; ++u) z[ax][u] = 0.0f;
 #pragma unroll
@@ -119,27 +121,44 @@ __global__ void __launch_bounds__(32 * kRegWarps) mg_vanka_reg(const RegVankaArg
     }
 }
 
-// inv [class][cell][np][npp] (float or bf16) -> out [class][np * np][cell], 32 x 32 tiles through shared
-// memory; cells on grid.x, which alone takes more than 65535 tiles of them
-template <typename W>
-__global__ void __launch_bounds__(256) vanka_columns(const W* __restrict__ in, float* __restrict__ out, int np, int npp,
+// The inverses by cell, [class][cell][np][npp] (zeros past np), to and from the
+// order of this sweep, [class][np * np][cell]: 32 x 32 tiles through shared
+// memory; cells on grid.x, which alone takes more than 65535 tiles of them.
+template <typename W, bool TO_COLUMNS>
+__global__ void __launch_bounds__(256) vanka_columns(const W* __restrict__ in, W* __restrict__ out, int np, int npp,
                                                      int n_cells, int n_classes) {
-  __shared__ float tile[32][33];
+  __shared__ W tile[32][33];
   const int c0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
+  const int width = TO_COLUMNS ? np : npp;                     // entries of a patch row: without or with the zeros
   for (int cls = blockIdx.z; cls < n_classes; cls += gridDim.z) {
-    const W* src = in + (long long)cls * n_cells * np * npp;
-    float* dst = out + (long long)cls * np * np * n_cells;
+    const long long by_cell = (long long)cls * n_cells * np * npp, by_entry = (long long)cls * np * np * n_cells;
     for (int j = threadIdx.y; j < 32; j += 8) {
-      const int c = c0 + j, e = e0 + threadIdx.x;
-      if (c < n_cells && e < np * np) tile[j][threadIdx.x] = (float)src[((long long)c * np + e / np) * npp + e % np];
+      const int c = c0 + (TO_COLUMNS ? j : threadIdx.x), e = e0 + (TO_COLUMNS ? threadIdx.x : j);
+      const int row = e / width, col = e % width;
+      if (c >= n_cells || e >= np * width) continue;
+      if (TO_COLUMNS) tile[j][threadIdx.x] = in[by_cell + ((long long)c * np + row) * npp + col];
+      else tile[threadIdx.x][j] = col < np ? in[by_entry + (long long)(row * np + col) * n_cells + c] : W(0.0f);
     }
     __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
-      const int e = e0 + j, c = c0 + threadIdx.x;
-      if (c < n_cells && e < np * np) dst[(long long)e * n_cells + c] = tile[threadIdx.x][j];
+      const int c = c0 + (TO_COLUMNS ? threadIdx.x : j), e = e0 + (TO_COLUMNS ? j : threadIdx.x);
+      if (c >= n_cells || e >= np * width) continue;
+      if (TO_COLUMNS) out[by_entry + (long long)e * n_cells + c] = tile[threadIdx.x][j];
+      else out[by_cell + ((long long)c * np + e / width) * npp + e % width] = tile[j][threadIdx.x];
     }
     __syncthreads();
   }
+}
+
+template <typename W>
+cudaError_t reorder(bool to_columns, const void* in, void* out, int np, int npp, int n_classes, long long n_cells) {
+  const int entries = np * (to_columns ? np : npp);
+  const dim3 grid((unsigned)((n_cells + 31) / 32), (entries + 31) / 32, std::min(n_classes, 65535)), block(32, 8);
+  const W* a = static_cast<const W*>(in);
+  W* b = static_cast<W*>(out);
+  if (to_columns) vanka_columns<W, true><<<grid, block>>>(a, b, np, npp, (int)n_cells, n_classes);
+  else vanka_columns<W, false><<<grid, block>>>(a, b, np, npp, (int)n_cells, n_classes);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -148,18 +167,21 @@ bool vanka_reg_eligible(int dim, int k, int nt) {
   return dim == 2 && k <= 2 && nt * (k + 1) * (k + 1) <= 18;
 }
 
-cudaError_t vanka_reg_columns(const void* inv, bool bf16, int np, int npp, int n_classes, long long n_cells, float** out) {
-  const size_t n = (size_t)n_classes * np * np * n_cells;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(out), n * sizeof(float));
+cudaError_t vanka_reg_reorder(bool to_columns, const void* in, bool bf16, int np, int npp, int n_classes,
+                              long long n_cells, void** out) {
+  const size_t n = (size_t)n_classes * n_cells * np * (to_columns ? np : npp);
+  *out = nullptr;
+  cudaError_t e = cudaMalloc(out, n * (bf16 ? sizeof(__nv_bfloat16) : sizeof(float)));
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)((n_cells + 31) / 32), (np * np + 31) / 32, std::min(n_classes, 65535)), block(32, 8);
-  if (bf16) vanka_columns<<<grid, block>>>(static_cast<const __nv_bfloat16*>(inv), *out, np, npp, (int)n_cells, n_classes);
-  else vanka_columns<<<grid, block>>>(static_cast<const float*>(inv), *out, np, npp, (int)n_cells, n_classes);
-  return cudaGetLastError();
+  e = bf16 ? reorder<__nv_bfloat16>(to_columns, in, *out, np, npp, n_classes, n_cells)
+           : reorder<float>(to_columns, in, *out, np, npp, n_classes, n_cells);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+  return e;
 }
 
-cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, const float* inv, const int* blk_cls,
-                             const int* blk_alpha, int n_blk, int n_classes, float omega, int trans, cudaStream_t s) {
+cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, const void* inv, bool bf16,
+                             const int* blk_cls, const int* blk_alpha, int n_blk, int n_classes, float omega, int trans,
+                             cudaStream_t s) {
   RegVankaArgs p;
   p.r = r;
   p.x = x;
@@ -183,11 +205,13 @@ cudaError_t launch_vanka_reg(const HostProblem& hp, const float* r, float* x, co
   const long long warps = (long long)grid.x * n_blk, room = 16 * sm_count();
   for (int split : {2, 3, 4, 6, 8})
     if (split <= hp.n_t * (hp.k + 1) && warps * split <= room) grid.z = split;
-#define SG_R(KK, TT)                                                   \
-  if (hp.dim == 2 && hp.k == KK && hp.n_t == TT) {                     \
-    if (trans) mg_vanka_reg<KK, TT, true><<<grid, block, 0, s>>>(p);   \
-    else mg_vanka_reg<KK, TT, false><<<grid, block, 0, s>>>(p);        \
-    return cudaGetLastError();                                         \
+#define SG_R(KK, TT)                                                                               \
+  if (hp.dim == 2 && hp.k == KK && hp.n_t == TT) {                                                 \
+    if (bf16 && trans) mg_vanka_reg<KK, TT, true, __nv_bfloat16><<<grid, block, 0, s>>>(p);        \
+    else if (bf16) mg_vanka_reg<KK, TT, false, __nv_bfloat16><<<grid, block, 0, s>>>(p);           \
+    else if (trans) mg_vanka_reg<KK, TT, true, float><<<grid, block, 0, s>>>(p);                   \
+    else mg_vanka_reg<KK, TT, false, float><<<grid, block, 0, s>>>(p);                             \
+    return cudaGetLastError();                                                                     \
   }
   SG_R(1, 1) SG_R(1, 2) SG_R(1, 3) SG_R(1, 4) SG_R(2, 1) SG_R(2, 2)
 #undef SG_R
