@@ -8,9 +8,14 @@
 // (450 unknowns; also once per Monte-Carlo call); this one is 29 launches,
 // bound by the serial chain through the pivot block.  Pivots are taken in
 // order: the operator's symmetric part is positive definite for an elliptic
-// coefficient.  A coefficient that is not may need exchanges, so the inverse
-// is checked against the matrix and the caller falls back to the pivoting
-// elimination when it fails.
+// coefficient.  A coefficient that is not may need exchanges, so the inverse X
+// of C is checked on a vector v > 0 and the caller falls back to the pivoting
+// elimination when |C (X v) - v| is above a bound times the largest entry of
+// |C| |X| v, the size of the terms that cancel there.  For FP64 levels the bound
+// is 8 roundings: elliptic operators of 126 to 2047 unknowns stay below 4, as
+// the pivoting elimination does, while indefinite ones (a negative mean
+// coefficient) that reach 10 to 1e5 have lost one to five digits against it.
+// FP32 levels, which store X to 2^-24, take 2^-32.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -78,15 +83,26 @@ __global__ void __launch_bounds__(256) coarse_step(const double* __restrict__ A,
   }
 }
 
-// y = A x, a warp per row
-__global__ void coarse_mv(const double* __restrict__ A, const double* __restrict__ x, double* __restrict__ y, int n) {
+// y = A x and ya = |A| xa, a warp per row
+__global__ void coarse_mv(const double* __restrict__ A, const double* __restrict__ x, const double* __restrict__ xa,
+                          double* __restrict__ y, double* __restrict__ ya, int n) {
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
-  double s = 0.0;
-  for (int q = lane; q < n; q += 32) s = fma(A[(size_t)row * n + q], x[q], s);
+  double s = 0.0, sa = 0.0;
+  for (int q = lane; q < n; q += 32) {
+    const double a = A[(size_t)row * n + q];
+    s = fma(a, x[q], s);
+    sa = fma(fabs(a), xa[q], sa);
+  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) y[row] = s;
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    sa += __shfl_xor_sync(0xffffffffu, sa, o);
+  }
+  if (lane == 0) {
+    y[row] = s;
+    ya[row] = sa;
+  }
 }
 
 template <typename T>
@@ -100,15 +116,15 @@ __global__ void coarse_store(const double* __restrict__ a, T* __restrict__ out, 
 cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int precision, void* out, bool& ok) {
   ok = false;
   const size_t nn = (size_t)n * n;
-  double* buf = nullptr;   // the matrix, two work buffers, three vectors, the flag
-  cudaError_t e = cudaMalloc(&buf, (3 * nn + 3 * (size_t)n + 1) * sizeof(double));
+  double* buf = nullptr;   // the matrix, two work buffers, five vectors, the flag
+  cudaError_t e = cudaMalloc(&buf, (3 * nn + 5 * (size_t)n + 1) * sizeof(double));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cudaSuccess;    // no room beside the level: the caller's way needs none
   }
-  double *A0 = buf, *w[2] = {buf + nn, buf + 2 * nn}, *v = buf + 3 * nn, *y = v + n, *z = y + n;
-  int* flag = reinterpret_cast<int*>(z + n);
-  std::vector<double> hv(n), hz(n);
+  double *A0 = buf, *w[2] = {buf + nn, buf + 2 * nn}, *v = buf + 3 * nn, *y = v + n, *ya = y + n, *z = ya + n, *za = z + n;
+  int* flag = reinterpret_cast<int*>(za + n);
+  std::vector<double> hv(n), hz(2 * (size_t)n);
   for (int i = 0; i < n; ++i) hv[i] = 1.0 + 0.5 * ((i * 37) % 101) / 101.0;
   e = cudaMemcpy(A0, C.data(), nn * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(v, hv.data(), n * sizeof(double), cudaMemcpyHostToDevice);
@@ -121,19 +137,19 @@ cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int preci
       coarse_step<<<grid, 256>>>(from, w[at], n, k0, flag);
       from = w[at];
     }
-    coarse_mv<<<(n + 7) / 8, 256>>>(from, v, y, n);
-    coarse_mv<<<(n + 7) / 8, 256>>>(A0, y, z, n);
+    coarse_mv<<<(n + 7) / 8, 256>>>(from, v, v, y, ya, n);
+    coarse_mv<<<(n + 7) / 8, 256>>>(A0, y, ya, z, za, n);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpy(hz.data(), z, n * sizeof(double), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(hz.data(), z, 2 * n * sizeof(double), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&singular, flag, sizeof(int), cudaMemcpyDeviceToHost);
-    // C (C^-1 v) = v to rounding, or the elimination lost it
-    double off = 0.0;
+    double off = 0.0, size = 0.0;
     bool finite = true;
     for (int i = 0; i < n; ++i) {
-      finite = finite && std::isfinite(hz[i]);
+      finite = finite && std::isfinite(hz[i]) && std::isfinite(hz[n + i]);
       off = std::max(off, std::fabs(hz[i] - hv[i]));
+      size = std::max(size, hz[n + i]);
     }
-    ok = e == cudaSuccess && !singular && finite && off <= 1e-9;
+    ok = e == cudaSuccess && !singular && finite && off <= (precision == kPrecF32 ? 0x1p-32 : 8 * 0x1p-52) * size;
     if (ok) {
       const int g = (int)std::min<size_t>((nn + 255) / 256, (size_t)sm_count() * 16);
       if (precision == kPrecF32) coarse_store<float><<<g, 256>>>(from, static_cast<float*>(out), (long long)nn);
