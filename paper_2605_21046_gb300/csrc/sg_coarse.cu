@@ -114,7 +114,8 @@ __global__ void coarse_store(const double* __restrict__ a, T* __restrict__ out, 
 }  // namespace
 
 cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int precision, void* out, bool& ok) {
-  ok = false;
+  ok = n == 0;              // a mesh without interior nodes has nothing to invert
+  if (ok) return cudaSuccess;
   const size_t nn = (size_t)n * n;
   double* buf = nullptr;   // the matrix, two work buffers, five vectors, the flag
   cudaError_t e = cudaMalloc(&buf, (3 * nn + 5 * (size_t)n + 1) * sizeof(double));

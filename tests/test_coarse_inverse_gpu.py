@@ -44,3 +44,19 @@ def test_indefinite_coarse_solve_keeps_its_digits(cuda, name):
         off = np.abs(C @ z[a][L.inner] - rhs).max()
         size = (np.abs(C) @ (np.abs(L.Ainv[mg.cls[a]]) @ np.abs(rhs))).max()
         assert off <= 64 * 2.0 ** -52 * size, off / size * 2.0 ** 52
+
+
+@pytest.mark.parametrize("prec", [sg.SG_PREC_FP64, sg.SG_PREC_FP32, sg.SG_PREC_BF16], ids=["fp64", "fp32", "bf16"])
+def test_set_up_without_interior_nodes(cuda, prec):
+    """A row of Q1 cells has boundary nodes only: set-up has nothing to invert,
+    and the operator is the identity."""
+    spec = dict(name="row", dim=2, cells=(4, 1), lo=(0.0, 0.0), hi=(1.0, 1.0), k=1, r=1, n_slabs=4, T=1.0, M=1, P=1,
+                coef=I.linear_sine_coef(1, 2, 0.1, [(1, 1)]))
+    ctx = sg.sg_setup_spec(spec)
+    sg.sg_mg_setup(ctx, prec)
+    assert sg.sg_mg_level_info(ctx, 0)["coarsest"] == 1
+    x = cuda.from_numpy(I.random_vector(spec)).cuda()
+    y = cuda.full_like(x, float("nan"))
+    sg.sg_apply(ctx, 0, x, y)
+    assert cuda.equal(x, y)
+    ctx.destroy()
