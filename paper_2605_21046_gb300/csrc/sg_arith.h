@@ -140,8 +140,9 @@ struct DW {
   }
   __device__ __forceinline__ static T neg(T a) { return {-a.h, -a.l}; }
   // Normalisation in three additions instead of TwoSum's six: exact when
-  // |l| <= |h|, and also when sums have cancelled h below l, because h is then
-  // a multiple of l's last place (both come from terms of the larger size).
+  // |l| <= |h|.  Where sums have cancelled h below l it loses at most 2^-24 |l|;
+  // l holds the roundings of the sums, 2^-24 of their terms, so that is within
+  // 2^-48 of the terms that cancelled, like the roundings of l itself.
   __device__ __forceinline__ static T fin(T a) {
     const float s = __fadd_rn(a.h, a.l);
     return {s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
