@@ -22,6 +22,7 @@
 #include <cmath>
 #include <vector>
 
+#include "sg_bounds.h"
 #include "sg_internal.h"
 
 namespace sg {
@@ -36,13 +37,15 @@ __global__ void __launch_bounds__(256) coarse_step(const double* __restrict__ A,
   __shared__ double P[kPiv][kPiv + 1], M[kTile][kPiv + 1], R[kTile][kPiv + 1], C[kPiv][kTile + 1];
   const int tid = threadIdx.x, r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile, kb = min(kPiv, n - k0);
   const int pi = tid / kPiv, pj = tid % kPiv;
+  const long long nn = (long long)n * n;
+  auto at = [&](long long r, long long c) { return SG_IN(r * n + c, nn, 511) ? A[r * n + c] : 0.0; };
   // the pivot block (padded with the identity), its rows and its columns in this tile
-  P[pi][pj] = pi < kb && pj < kb ? A[(size_t)(k0 + pi) * n + k0 + pj] : (pi == pj ? 1.0 : 0.0);
+  P[pi][pj] = pi < kb && pj < kb ? at(k0 + pi, k0 + pj) : (pi == pj ? 1.0 : 0.0);
   for (int e = tid; e < kTile * kPiv; e += 256) {
     const int a = e / kPiv, q = e % kPiv;
-    R[a][q] = r0 + a < n && q < kb ? A[(size_t)(r0 + a) * n + k0 + q] : 0.0;
+    R[a][q] = r0 + a < n && q < kb ? at(r0 + a, k0 + q) : 0.0;
     const int cq = e / kTile, cc = e % kTile;
-    C[cq][cc] = cq < kb && c0 + cc < n ? A[(size_t)(k0 + cq) * n + c0 + cc] : 0.0;
+    C[cq][cc] = cq < kb && c0 + cc < n ? at(k0 + cq, c0 + cc) : 0.0;
   }
   __syncthreads();
   for (int q = 0; q < kPiv; ++q) {
@@ -75,11 +78,11 @@ __global__ void __launch_bounds__(256) coarse_step(const double* __restrict__ A,
     if (ck >= 0 && ck < kb) {
       v = -M[a][ck];
     } else {
-      v = rk >= 0 && rk < kb ? 0.0 : A[(size_t)r * n + c];
+      v = rk >= 0 && rk < kb ? 0.0 : at(r, c);
 #pragma unroll
       for (int q = 0; q < kPiv; ++q) v = fma(-M[a][q], C[q][b], v);
     }
-    out[(size_t)r * n + c] = v;
+    if (SG_IN((long long)r * n + c, nn, 512)) out[(size_t)r * n + c] = v;
   }
 }
 
@@ -90,7 +93,7 @@ __global__ void coarse_mv(const double* __restrict__ A, const double* __restrict
   if (row >= n) return;
   double s = 0.0, sa = 0.0;
   for (int q = lane; q < n; q += 32) {
-    const double a = A[(size_t)row * n + q];
+    const double a = SG_IN((long long)row * n + q, (long long)n * n, 513) ? A[(size_t)row * n + q] : 0.0;
     s = fma(a, x[q], s);
     sa = fma(fabs(a), xa[q], sa);
   }
@@ -164,3 +167,5 @@ cudaError_t coarse_inverse_device(const std::vector<double>& C, int n, int preci
 }
 
 }  // namespace sg
+
+SG_BOUNDS_FETCH(bounds_fetch_coarse)

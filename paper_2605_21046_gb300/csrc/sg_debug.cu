@@ -17,6 +17,7 @@ cudaError_t bounds_fetch_factor(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_debug(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_vanka_tc(BoundsRecord* out, bool clear);
 cudaError_t bounds_fetch_vanka_reg(BoundsRecord* out, bool clear);
+cudaError_t bounds_fetch_coarse(BoundsRecord* out, bool clear);
 }  // namespace sg
 
 namespace {
@@ -52,7 +53,7 @@ sg_status sg_debug_bounds(int* enabled, unsigned int* count, int* site, long lon
   cudaError_t (*const fetch[])(sg::BoundsRecord*, bool) = {
       sg::bounds_fetch_apply_f64, sg::bounds_fetch_apply_dw, sg::bounds_fetch_apply_f32,
       sg::bounds_fetch_mg,        sg::bounds_fetch_factor,   sg::bounds_fetch_debug, sg::bounds_fetch_vanka_tc,
-      sg::bounds_fetch_diag, sg::bounds_fetch_vanka_reg};
+      sg::bounds_fetch_diag, sg::bounds_fetch_vanka_reg, sg::bounds_fetch_coarse};
   for (auto f : fetch) {
     sg::BoundsRecord r;
     if (f(&r, true) != cudaSuccess) return fail(SG_ERR_CUDA, "sg_debug_bounds: reading a record failed");

@@ -574,10 +574,10 @@ __device__ __forceinline__ void transfer_load(const TransferParams<T>& p, const 
 }
 
 // One 1D pass along x or y of `rows` output rows: DIR 0 out[row][c] = sum_k w in[row][idx[o0 + c] - lo],
-// DIR 1 out[row][c] = sum_k w in[idx[o0 + row] - lo][c]; put(row, column, value).
+// DIR 1 out[row][c] = sum_k w in[idx[o0 + row] - lo][c]; put(row, column, value).  n_in input rows.
 template <typename T, int W, int DIR, class Put>
 __device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, int cb, int rows, const int* idx,
-                                              const T* w, int n_list, int o0, int lo, Put put) {
+                                              const T* w, int n_list, int o0, int lo, int n_in, Put put) {
   const int par = kTransferThreads / cb;                       // cb columns x par rows at a time
   const int c0 = threadIdx.x % cb, r0 = threadIdx.x / cb;
   if (r0 >= par) return;
@@ -593,15 +593,18 @@ __device__ __forceinline__ void transfer_pass(const T* in, int pitch, int cols, 
       for (int r = r0; r < rows; r += par) {
         T s = T(0);
 #pragma unroll
-        for (int k = 0; k < W; ++k) s = fma(wt[k], in[r * pitch + at[k]], s);
+        for (int k = 0; k < W; ++k)
+          if (SG_IN(at[k], pitch, 504)) s = fma(wt[k], in[r * pitch + at[k]], s);
         put(r, c, s);
       }
     } else {
       for (int r = r0; r < rows; r += par) {
         T s = T(0);
 #pragma unroll
-        for (int k = 0; k < W; ++k)
-          s = fma(__ldg(w + k * n_list + o0 + r), in[(__ldg(idx + k * n_list + o0 + r) - lo) * pitch + c], s);
+        for (int k = 0; k < W; ++k) {
+          const int at = __ldg(idx + k * n_list + o0 + r) - lo;
+          if (SG_IN(at, n_in, 505)) s = fma(__ldg(w + k * n_list + o0 + r), in[at * pitch + c], s);
+        }
         put(r, c, s);
       }
     }
@@ -617,11 +620,11 @@ __global__ void __launch_bounds__(kTransferThreads) mg_restrict(const TransferPa
   transfer_load<T, W, LARGE>(p, t, S0);
   __syncthreads();
   const int ncx = p.no[0], nc = LARGE ? t.ni : ncx;
-  transfer_pass<T, W, 0>(S0, t.cntx, nc, p.cb_out, t.cnt, p.idx[0], p.w[0], ncx, t.i0, t.lox,
+  transfer_pass<T, W, 0>(S0, t.cntx, nc, p.cb_out, t.cnt, p.idx[0], p.w[0], ncx, t.i0, t.lox, t.cnt,
                          [&](int r, int c, T v) { S1[r * nc + c] = v; });
   __syncthreads();
   const long long o0 = (long long)t.v * p.n_out + ((long long)t.jz * p.no[1] + t.j0) * ncx + t.i0;
-  transfer_pass<T, W, 1>(S1, nc, nc, p.cb_out, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo, [&](int r, int c, T v) {
+  transfer_pass<T, W, 1>(S1, nc, nc, p.cb_out, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo, t.cnt, [&](int r, int c, T v) {
     const long long o = o0 + (long long)r * ncx + c;
     if (!SG_IN(o, p.lim_out, 502)) return;
     p.out[o] = v;
@@ -641,10 +644,10 @@ __global__ void __launch_bounds__(kTransferThreads) mg_prolong(const TransferPar
   transfer_load<T, W, LARGE>(p, t, S0);
   __syncthreads();
   const int nfx = p.no[0];
-  transfer_pass<T, W, 1>(S0, t.cntx, t.cntx, p.cb_in, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo,
+  transfer_pass<T, W, 1>(S0, t.cntx, t.cntx, p.cb_in, t.nj, p.idx[1], p.w[1], p.no[1], t.j0, t.lo, t.cnt,
                          [&](int r, int c, T v) { S1[r * t.cntx + c] = v; });
   __syncthreads();
-  transfer_pass<T, W, 0>(S1, t.cntx, t.ni, p.cb_out, t.nj, p.idx[0], p.w[0], nfx, t.i0, t.lox,
+  transfer_pass<T, W, 0>(S1, t.cntx, t.ni, p.cb_out, t.nj, p.idx[0], p.w[0], nfx, t.i0, t.lox, t.nj,
                          [&](int r, int c, T v) { S2[r * t.ni + c] = v; });
   __syncthreads();
   // x += S2, r = b inside (whole rows of a tile are contiguous), with the loads of a batch in flight together
@@ -690,7 +693,8 @@ __global__ void __launch_bounds__(32 * kCoarseRows) mg_coarse(const T* __restric
                                                               const T* __restrict__ inv, const int* __restrict__ blk_cls,
                                                               const int* __restrict__ blk_alpha,
                                                               const long long* __restrict__ inner, int n_int, int n_t,
-                                                              long long n_x, int trans) {
+                                                              long long n_x, int trans, long long lim_vec,
+                                                              long long lim_inv) {
   extern __shared__ __align__(16) unsigned char sm[];
   T* bs = reinterpret_cast<T*>(sm);                            // [mode][n_int]
   const int blk = blockIdx.y;
@@ -703,7 +707,7 @@ __global__ void __launch_bounds__(32 * kCoarseRows) mg_coarse(const T* __restric
   for (int i = threadIdx.x; i < n_int; i += blockDim.x) {
     const long long at = __ldg(inner + i);
 #pragma unroll
-    for (int u = 0; u < kCoarseModes; ++u) bs[u * n_int + i] = base[u] >= 0 ? __ldg(b + base[u] + at) : T(0);
+    for (int u = 0; u < kCoarseModes; ++u) bs[u * n_int + i] = base[u] >= 0 && SG_IN(base[u] + at, lim_vec, 506) ? __ldg(b + base[u] + at) : T(0);
   }
   __syncthreads();
   const T* M = inv + (long long)__ldg(blk_cls + blk) * n_int * n_int;
@@ -715,7 +719,7 @@ __global__ void __launch_bounds__(32 * kCoarseRows) mg_coarse(const T* __restric
   T s[kCoarseModes] = {};
 #pragma unroll 4
   for (int q = lane; q < n_int; q += 32) {
-    const T w = __ldg(row + q * step);
+    const T w = SG_IN(row - inv + q * step, lim_inv, 507) ? __ldg(row + q * step) : T(0);
 #pragma unroll
     for (int u = 0; u < kCoarseModes; ++u) s[u] = fma(w, bs[u * n_int + q], s[u]);
   }
@@ -723,7 +727,8 @@ __global__ void __launch_bounds__(32 * kCoarseRows) mg_coarse(const T* __restric
   for (int u = 0; u < kCoarseModes; ++u) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-    if (lane == 0 && base[u] >= 0) x[base[u] + __ldg(inner + i)] = s[u];
+    const long long at = base[u] + __ldg(inner + i);
+    if (lane == 0 && base[u] >= 0 && SG_IN(at, lim_vec, 508)) x[at] = s[u];
   }
 }
 
@@ -1355,7 +1360,8 @@ cudaError_t issue_vcycle(MG& mg, int l, cudaStream_t s, int trans) {
     const size_t smem = (size_t)kCoarseModes * L.n_int * sizeof(T);
     mg_coarse<T><<<dim3((L.n_int + kCoarseRows - 1) / kCoarseRows, mg.n_blk), 32 * kCoarseRows, smem, s>>>(
         static_cast<const T*>(L.d_b), static_cast<T*>(L.d_x), static_cast<const T*>(L.d_inv), mg.d_blk_cls,
-        mg.d_blk_alpha, reinterpret_cast<const long long*>(L.d_inner), L.n_int, L.hp.n_t, L.hp.n_x, trans);
+        mg.d_blk_alpha, reinterpret_cast<const long long*>(L.d_inner), L.n_int, L.hp.n_t, L.hp.n_x, trans,
+        (long long)V * L.hp.n_x, (long long)mg.n_classes * L.n_int * L.n_int);
     return cudaGetLastError();
   }
   cudaError_t e;

@@ -130,21 +130,26 @@ __global__ void __launch_bounds__(256) vanka_columns(const W* __restrict__ in, W
   __shared__ W tile[32][33];
   const int c0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
   const int width = TO_COLUMNS ? np : npp;                     // entries of a patch row: without or with the zeros
+  const long long n_cell = (long long)n_classes * n_cells * np * npp, n_entry = (long long)n_classes * np * np * n_cells;
   for (int cls = blockIdx.z; cls < n_classes; cls += gridDim.z) {
     const long long by_cell = (long long)cls * n_cells * np * npp, by_entry = (long long)cls * np * np * n_cells;
     for (int j = threadIdx.y; j < 32; j += 8) {
       const int c = c0 + (TO_COLUMNS ? j : threadIdx.x), e = e0 + (TO_COLUMNS ? threadIdx.x : j);
       const int row = e / width, col = e % width;
       if (c >= n_cells || e >= np * width) continue;
-      if (TO_COLUMNS) tile[j][threadIdx.x] = in[by_cell + ((long long)c * np + row) * npp + col];
-      else tile[threadIdx.x][j] = col < np ? in[by_entry + (long long)(row * np + col) * n_cells + c] : W(0.0f);
+      const long long at = TO_COLUMNS ? by_cell + ((long long)c * np + row) * npp + col
+                                      : by_entry + (long long)(row * np + col) * n_cells + c;
+      const W v = col < np && SG_IN(at, TO_COLUMNS ? n_cell : n_entry, 804) ? in[at] : W(0.0f);
+      if (TO_COLUMNS) tile[j][threadIdx.x] = v;
+      else tile[threadIdx.x][j] = v;
     }
     __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
       const int c = c0 + (TO_COLUMNS ? threadIdx.x : j), e = e0 + (TO_COLUMNS ? j : threadIdx.x);
       if (c >= n_cells || e >= np * width) continue;
-      if (TO_COLUMNS) out[by_entry + (long long)e * n_cells + c] = tile[threadIdx.x][j];
-      else out[by_cell + ((long long)c * np + e / width) * npp + e % width] = tile[j][threadIdx.x];
+      const long long at = TO_COLUMNS ? by_entry + (long long)e * n_cells + c
+                                      : by_cell + ((long long)c * np + e / width) * npp + e % width;
+      if (SG_IN(at, TO_COLUMNS ? n_entry : n_cell, 805)) out[at] = TO_COLUMNS ? tile[threadIdx.x][j] : tile[j][threadIdx.x];
     }
     __syncthreads();
   }
