@@ -310,8 +310,9 @@ cudaError_t launch_apply(const HostProblem& hp, const LaunchShape& ls, const App
   // The cell kernel needs y's start only before its first reduction, so it may
   // begin while the start pass runs: its tables, gathers and first chunk hide
   // the pass and the gap between two launches (45x37 Q2 dG(2) 36.9 -> 34.9 us,
-  // 64^2 Q2 149 -> 147; 8x8 Q1 14.4 -> 11.4, where the caller's host time is next).  Inside a capture the kernels are already back to back, and a
-  // plain edge is recorded.
+  // 64^2 Q2 149 -> 147; 8x8 Q1 14.3 -> 12.4 from Python, whose own time varies by
+  // 2 us with the process; 10.3 from C).  Inside a capture the kernels are already
+  // back to back, and a plain edge is recorded.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(stream, &cap);
   if (e != cudaSuccess) return e;

@@ -12,7 +12,7 @@
 // of C is checked on a vector v > 0 and the caller falls back to the pivoting
 // elimination when |C (X v) - v| is above a bound times the largest entry of
 // |C| |X| v, the size of the terms that cancel there.  For FP64 levels the bound
-// is 8 roundings: elliptic operators of 126 to 2047 unknowns stay below 4, as
+// is 8 roundings: elliptic operators of 450 to 2000 unknowns stay below 4, as
 // the pivoting elimination does, while indefinite ones (a negative mean
 // coefficient) that reach 10 to 1e5 have lost one to five digits against it.
 // FP32 levels, which store X to 2^-24, take 2^-32.

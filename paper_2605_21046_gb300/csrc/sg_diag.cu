@@ -16,7 +16,7 @@
 //
 // The cell work is about 750 FMAs per vector (3D Q2).  Held in shared memory it
 // was bound by that memory's wavefronts (28 accesses per point and row) and
-// took 295 us on 32^3 Q2 with 20 rows in FP32; this kernel takes about 60 us
+// took 295 us on 32^3 Q2 with 20 rows in FP32; this kernel takes 78 us
 // (the V-cycle went from 1.46 to 0.97 ms with bf16 factors, 64^2 Q2 with 35
 // rows from 0.254 to 0.201 ms).
 #include <cuda_runtime.h>

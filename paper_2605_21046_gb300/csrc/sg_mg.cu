@@ -1897,8 +1897,12 @@ sg_status mg_build(const HostProblem& fine, int precision, int nu, double omega,
       L.ffma_chunk = L.vanka_chunk;
       if ((e = prepare_vanka(L.hp.dim, L.hp.k, L.hp.n_t, precision == kPrecF32, mg.bf16)) != cudaSuccess) break;
       if (mg.bf16 && (e = prepare_vanka_tc(L.hp.dim, L.hp.k, L.hp.n_t)) != cudaSuccess) break;
-      // FP32 vectors and small 2D patches: the register sweep, always the fastest there
-      // (V-cycle with it and with the tuned FFMA or tensor-core sweep: 64^2 Q2, 35 rows 0.115 and 0.158 ms; 128^2 Q2, 70 rows 0.46 and 0.70)
+      // FP32 vectors and small 2D patches: the register sweep, untimed.  V-cycle with it
+      // and with the best of the other sweeps over their chunks, ms: 32^2 Q2 dG(1), 35 rows
+      // 0.064 / 0.078; 64^2, 165 rows 0.289 / 0.478; 256^2, 35 rows FP32 0.970 / 1.288, bf16
+      // 0.946 / 1.133 (tensor cores), of 35 diagonal classes 2.24 / 17.7; 512^2, 35 rows 3.48 /
+      // 4.74; 1024^2, 2 rows 1.69 / 2.78; Q1 dG(0) 1024^2, 35 rows 1.90 / 3.27; Q1 dG(3)
+      // 512^2, 35 rows 2.30 / 3.38: faster on each of the 40 shapes measured in that range.
       if (precision == kPrecF32 && vanka_reg_eligible(L.hp.dim, L.hp.k, L.hp.n_t)) {
         // its order takes the place of the order by cell; without room for both at once the
         // level keeps that one, and its sweep is timed like the others

@@ -514,7 +514,6 @@ cudaError_t vanka_tc_wait_probe(unsigned int polls, int* status_out) {
   return e;
 }
 
-// slots of a tile rounded up to 16: the column pitch of one split term
 // columns of a split term: a multiple of 8, so that both terms make an N of a multiple of 16
 static int tc_slot_pitch(int tile_slots) { return (tile_slots + 7) / 8 * 8; }
 
